@@ -144,8 +144,8 @@ typedef struct aes_batch_plan aes_batch_plan;
 
 /* Builds a reusable plan: validates every descriptor (AES_ERR_ARG /
  * AES_ERR_ALIGN), groups messages by direction and key size, tiles the
- * flattened blocks (one tile = 128 * blocks_per_thread blocks, taken by one
- * warp; CTAs of `threads` threads; blocks_per_thread 1, 2, 4 or 8, with 8
+ * flattened blocks (one tile = 128 * blocks_per_thread blocks, at most 512, taken
+ * by one warp, or in parts by several where there are few; CTAs of `threads` threads; blocks_per_thread 1, 2, 4 or 8, with 8
  * needing threads <= 512; 0, 0 = 1024, 2) and uploads the tile table, message table and every context's two
  * schedules to one device allocation on the current device (cudaMalloc,
  * synchronous).  msgs and ctxs are HOST arrays, read during the call only.
@@ -153,8 +153,8 @@ typedef struct aes_batch_plan aes_batch_plan;
 aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx,
                                       int threads, int blocks_per_thread);
 
-/* Launches a plan on `stream`: resets the plan's tile counters, then one
- * persistent kernel (one CTA per SM; its warps take tiles independently).  in_base/out_base: device buffers of
+/* Launches a plan on `stream`: resets the plan's tile counters (a batch with no
+ * more parts than warps needs none), then one persistent kernel (one CTA per SM; its warps take tiles independently).  in_base/out_base: device buffers of
  * in_bytes/out_bytes bytes that must cover every message (AES_ERR_ARG).  Two
  * launches of the same plan must not run concurrently (they share its tile
  * counter); stream-ordered repeats are fine. */
@@ -175,7 +175,7 @@ void aes_batch_plan_free(aes_batch_plan* plan);
 
 /* One-shot batch: plan tables in stream-ordered scratch (cudaMallocAsync /
  * cudaFreeAsync on `stream`), one launch with 1024 threads x 2 blocks per
- * tile.  Same arguments and rules as the plan calls.  The tables are uploaded
+ * thread, tiles of 512 blocks (2048 for batches above 2^23 blocks).  Same arguments and rules as the plan calls.  The tables are uploaded
  * from a host copy that is freed when the call returns, so a stream that is
  * being captured into a CUDA graph is refused (AES_ERR_STATE); for graphs use
  * a plan and aes_batch_plan_launch_graph. */
@@ -192,7 +192,7 @@ int aes_ecb_batch(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* c
  *    pool.  The array exists on every GPU that loads the library, until exit.
  *  - A batch whose tables exceed 8 MiB (512 bytes per key context, 32 bytes per
  *    message, 4 bytes per 2048-block tile, plus 256) is rejected with
- *    AES_ERR_ARG; the 10,000-message, 10,000-key batch needs about 5.6 MiB.
+ *    AES_ERR_ARG (the tiles are smaller where the tables leave room); the 10,000-message, 10,000-key batch needs about 5.6 MiB.
  *  - The first call in each CUDA context (normally once per device, in its
  *    primary context) looks up the array's device address there
  *    (cudaGetSymbolAddress) and keeps it for that context.

@@ -12,15 +12,15 @@
 //    gets a slot holding its 4*(Nr+1)-word schedule.  Everything sits in one
 //    device buffer, uploaded once per plan.
 //  * Kernel.  One CTA per SM holds the shared-memory tables of aes_rounds.cuh.
-//    Each *warp* starts on a fixed tile, then takes tiles from its
+//    Each *warp* starts on a fixed unit (a tile, or a part of one where there are
+//    fewer tiles than warps to share them), then takes units from its
 //    direction's atomic counter on its own, so the dependent loads at the
-//    start of one warp's tile overlap the other warps' lookups; the CTA meets
-//    at a barrier only to swap its tables from the encryption to the
-//    decryption set, once.  A block finds its message
-//    by binary search over the tile's message range (none when the tile lies
-//    in one message); a warp whose tile lies in one message stages that
-//    message's schedule in its shared-memory key slot, other tiles read keys
-//    from global memory through L1.  The round count is a run-time loop bound,
+//    start of one warp's unit overlap the other warps' lookups; the CTA meets
+//    at a barrier only to swap its tables from one direction's set to the
+//    other's, once at most.  A warp whose unit lies in one message stages that
+//    message's schedule in its shared-memory key slot; in other units every block
+//    finds its message from the starts of the next 32, and keys come from
+//    global memory through L1.  The round count is a run-time loop bound,
 //    so one compact body per direction serves all key sizes.
 #include <cuda_runtime.h>
 
@@ -40,25 +40,41 @@ namespace gbaes {
 
 constexpr uint32_t kPlanTileMax = 512;  // largest tile of a batch plan, in blocks
 
-// A tile inside one message m (the common case): blocks [tb0, tb0 + n) of the
-// group's block space map to consecutive blocks of m, processed 32*BPT at a
-// time (lane l, slot b -> block it + 32b + l, so every load and store
+__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
+constexpr uint32_t kNoBoundary = 0x7fffffffu;
+
+// Starts of the messages after `base`, relative to tb0: lane l gets message
+// base + 1 + l's (kNoBoundary past the group's last message or far away; 0 for
+// any start at or before tb0).  One coalesced load tells a warp where 32
+// messages begin.
+__device__ __forceinline__ uint32_t load_starts(const BatchArgs& a, const GroupDev& G, uint32_t base, uint64_t tb0,
+                                                uint32_t lane) {
+    const uint32_t m = base + 1u + lane;
+    if (m >= G.msg_end || m < base) return kNoBoundary;
+    const uint64_t s = __ldg((const unsigned long long*)(a.msgs + m));
+    if (s <= tb0) return 0u;
+    return s - tb0 < kNoBoundary ? (uint32_t)(s - tb0) : kNoBoundary;
+}
+
+// n consecutive blocks from tb0 inside one message m (the common case: 97.5% of
+// the 512-block tiles of a batch of 10,000 messages, 16 B - 4 MiB), processed
+// 32*BPT at a time (lane l, slot b -> block it + 32b + l, so every load and store
 // instruction of the warp covers 512 contiguous bytes).  The descriptor is
 // read once and m's schedule is staged in the warp's shared-memory key slot:
 // one parallel load instead of a dependent global load per round, issued once
 // the first data loads are in flight so that the two overlap.  Lanes past the
 // end compute on zeros and store nothing, so the warp stays converged.
 template <bool DEC, int BPT>
-__device__ __forceinline__ void single_message_tile(const BatchArgs& a, const GroupDev& G, uint32_t m, uint64_t tb0,
-                                                    uint32_t lane, uint32_t L0, uint32_t L1, uint32_t kslot) {
+__device__ __forceinline__ void single_message_unit(const BatchArgs& a, const GroupDev& G, uint32_t m, uint64_t tb0,
+                                                    uint32_t n, uint32_t lane, uint32_t L0, uint32_t L1,
+                                                    uint32_t kslot) {
     const uint4* mp = (const uint4*)(a.msgs + m);
     const uint4 q0 = __ldg(mp);
     const uint4 q1 = __ldg(mp + 1);
     const uint64_t off = tb0 - (((uint64_t)q0.y << 32) | q0.x);  // tb0 - blk_start
     const uint4* in = a.in + ((((uint64_t)q0.w << 32) | q0.z) + off);
     uint4* out = a.out + ((((uint64_t)q1.y << 32) | q1.x) + off);
-    const uint64_t left = G.blocks - tb0;
-    const uint32_t n = left < a.tile_blocks ? (uint32_t)left : a.tile_blocks;
     for (uint32_t it = 0; it < n; it += 32u * BPT) {
         uint32_t s[BPT][4];
 #pragma unroll
@@ -70,7 +86,7 @@ __device__ __forceinline__ void single_message_tile(const BatchArgs& a, const Gr
             s[b][2] = v.z;
             s[b][3] = v.w;
         }
-        if (it == 0) {  // (every lane has left the previous tile: the warp met at the tile-index shuffle)
+        if (it == 0) {  // (every lane has left the previous unit: the warp met at the unit-index shuffle)
             if (lane < (uint32_t)G.nr + 1u) {
                 const uint4 k = __ldg(a.keys + (uint64_t)q1.z * (kSlotWords / 4) + lane);
                 asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(kslot + 16u * lane), "r"(k.x),
@@ -88,75 +104,96 @@ __device__ __forceinline__ void single_message_tile(const BatchArgs& a, const Gr
     }
 }
 
-// A tile that crosses message boundaries (messages m_lo..m_hi, m_lo < m_hi):
-// each block finds its message by binary search over that range and reads its
-// round keys from global memory through L1.  The states of one thread may
-// belong to different messages: each carries its own key pointer, so the
-// warp runs one interleaved cipher over all of them (no divergent per-block
-// ciphers at a message boundary).
+// n consecutive blocks from tb0 that cross message boundaries, the first of them
+// in message m; `starts`: load_starts of a message at most 32 before the next
+// boundary.  Each block finds its message from the window of starts: a ballot
+// counts those a pass leaves behind, an OR over the warp marks the blocks at which
+// a message begins, and a lane's message is the one of block 0 plus the marks up
+// to the lane.  (A binary search per block took five or more dependent loads;
+// with the finer units of schedule_batch, the kernel's time for 2,000 messages of
+// 16 B - 16 KiB went from 33 to 14 us in a plan of 1024 x 2 and from 199 to 15 us in
+// a one-shot call.)  The states of one thread may belong to different messages:
+// each reads its own round keys from global memory through L1, where the
+// schedule's second line is fetched ahead, and the warp runs one interleaved
+// cipher over all of them (no divergent per-block ciphers at a boundary).
 template <bool DEC, int BPT>
-__device__ __forceinline__ void mixed_tile(const BatchArgs& a, const GroupDev& G, uint32_t m_lo, uint32_t m_hi,
-                                           uint64_t tb0, uint32_t lane, uint32_t L0, uint32_t L1) {
-    for (uint32_t it = 0; it < a.tile_blocks; it += 32u * BPT) {
+__device__ __forceinline__ void mixed_unit(const BatchArgs& a, const GroupDev& G, uint32_t m, uint32_t starts,
+                                           uint64_t tb0, uint32_t n, uint32_t lane, uint32_t L0, uint32_t L1) {
+    uint32_t wlast = __shfl_sync(0xffffffffu, starts, 31);  // the window's last entry
+    for (uint32_t it = 0; it < n; it += 32u * BPT) {
         uint32_t s[BPT][4];
         uint64_t oidx[BPT];
-        const uint4* kp[BPT];
+        uint32_t slot[BPT];
         bool ok[BPT];
 #pragma unroll
         for (int b = 0; b < BPT; ++b) {
-            const uint64_t gb = tb0 + it + 32u * b + lane;
-            ok[b] = gb < G.blocks && it + 32u * b + lane < a.tile_blocks;
+            const uint32_t g0 = it + 32u * b;
+            if (wlast <= g0 + 32u) {  // the window must reach past these blocks
+                starts = load_starts(a, G, m, tb0, lane);
+                wlast = __shfl_sync(0xffffffffu, starts, 31);
+            }
+            const uint32_t marks =
+                __reduce_or_sync(0xffffffffu, starts > g0 && starts < g0 + 32u ? 1u << (starts - g0) : 0u);
+            const uint32_t own = m + __popc(marks & (0xffffffffu >> (31u - lane)));
+            m += __popc(__ballot_sync(0xffffffffu, starts > g0 && starts <= g0 + 32u));
+            ok[b] = g0 + lane < n;
             uint4 v = make_uint4(0, 0, 0, 0);
-            kp[b] = nullptr;
+            slot[b] = 0;
             oidx[b] = 0;
             if (ok[b]) {
-                uint32_t lo = m_lo, hi = m_hi;  // largest m in [m_lo, m_hi] with blk_start[m] <= gb
-                while (lo < hi) {
-                    const uint32_t mid = (lo + hi + 1) >> 1;
-                    if (__ldg((const unsigned long long*)(a.msgs + mid)) <= gb)
-                        lo = mid;
-                    else
-                        hi = mid - 1;
-                }
-                const uint4* mp = (const uint4*)(a.msgs + lo);
+                const uint4* mp = (const uint4*)(a.msgs + own);
                 const uint4 r0 = __ldg(mp);
                 const uint4 r1 = __ldg(mp + 1);
-                const uint64_t blk_start = ((uint64_t)r0.y << 32) | r0.x;
-                const uint64_t in_blk = ((uint64_t)r0.w << 32) | r0.z;
-                const uint64_t out_blk = ((uint64_t)r1.y << 32) | r1.x;
-                const uint64_t off = gb - blk_start;
-                v = ld_stream(a.in + in_blk + off);
-                oidx[b] = out_blk + off;
-                kp[b] = a.keys + (uint64_t)r1.z * (kSlotWords / 4);
+                const uint64_t off = tb0 + g0 + lane - (((uint64_t)r0.y << 32) | r0.x);
+                v = ld_stream(a.in + ((((uint64_t)r0.w << 32) | r0.z) + off));
+                oidx[b] = (((uint64_t)r1.y << 32) | r1.x) + off;
+                slot[b] = r1.z;
+                prefetch_l1(a.keys + (uint64_t)r1.z * (kSlotWords / 4) + 8);
             }
             s[b][0] = v.x;
             s[b][1] = v.y;
             s[b][2] = v.z;
             s[b][3] = v.w;
         }
-        if (!ok[0]) return;  // blocks only increase: nothing left in this tile for this lane
+        if (ok[0]) {  // (else this lane's blocks are all past the end)
 #pragma unroll
-        for (int b = 1; b < BPT; ++b)
-            if (!ok[b]) kp[b] = kp[0];  // (past the end: computes on zeros with a valid key, stores nothing)
-        cipher_rt<DEC, BPT>(s, StateKeys<BPT>{kp}, G.nr, L0, L1);
+            for (int b = 1; b < BPT; ++b)
+                if (!ok[b]) slot[b] = slot[0];  // (past the end: computes on zeros with a valid key, stores nothing)
+            cipher_rt<DEC, BPT>(s, StateKeys<BPT, kSlotWords / 4>{a.keys, slot}, G.nr, L0, L1);
 #pragma unroll
-        for (int b = 0; b < BPT; ++b)
-            if (ok[b]) __stcs(a.out + oidx[b], make_uint4(s[b][0], s[b][1], s[b][2], s[b][3]));
+            for (int b = 0; b < BPT; ++b)
+                if (ok[b]) __stcs(a.out + oidx[b], make_uint4(s[b][0], s[b][1], s[b][2], s[b][3]));
+        }
+        __syncwarp();
     }
 }
 
-// One warp's tile t of group G: tile_blocks consecutive blocks of the group's
-// block space (fewer in the group's last tile).
+// Unit u of group G: part u mod 2^split of tile u >> split (tile_blocks
+// consecutive blocks of the group's block space, fewer in the group's last one).
 template <bool DEC, int BPT>
-__device__ __forceinline__ void batch_warp_tile(const BatchArgs& a, const GroupDev& G, uint32_t t, uint32_t lane,
+__device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupDev& G, uint32_t u, uint32_t lane,
                                                 uint32_t L0, uint32_t L1, uint32_t kslot) {
-    const uint64_t tb0 = (uint64_t)(t - G.tile_start) * a.tile_blocks;
+    const uint32_t t = u >> a.split;
+    const uint32_t part = a.tile_blocks >> a.split;
+    const uint64_t tb0 = (uint64_t)(t - G.tile_start) * a.tile_blocks + (u & ((1u << a.split) - 1u)) * part;
+    if (tb0 >= G.blocks) return;
+    const uint64_t left = G.blocks - tb0;
+    const uint32_t n = left < part ? (uint32_t)left : part;
     const uint32_t m_lo = a.tile_msg[t];
     const uint32_t m_hi = (t + 1 < G.tile_end) ? a.tile_msg[t + 1] : G.msg_end - 1;
-    if (m_lo == m_hi)
-        single_message_tile<DEC, BPT>(a, G, m_lo, tb0, lane, L0, L1, kslot);
+    uint32_t m = m_lo, starts = kNoBoundary;
+    if (m_lo != m_hi) {
+        for (;;) {  // find tb0's message; the starts after it stay in the window
+            starts = load_starts(a, G, m, tb0, lane);
+            const uint32_t passed = __popc(__ballot_sync(0xffffffffu, starts == 0u));
+            m += passed;
+            if (passed < 32u) break;
+        }
+    }
+    if (!__any_sync(0xffffffffu, starts != 0u && starts < n))
+        single_message_unit<DEC, BPT>(a, G, m, tb0, n, lane, L0, L1, kslot);
     else
-        mixed_tile<DEC, BPT>(a, G, m_lo, m_hi, tb0, lane, L0, L1);
+        mixed_unit<DEC, BPT>(a, G, m, starts, tb0, n, lane, L0, L1);
 }
 
 // Group table staged in shared memory (read with a runtime index per tile).
@@ -175,12 +212,15 @@ __device__ __forceinline__ GroupDev load_group(uint32_t gaddr, int g) {
     return G;
 }
 
-// Tiles [0, E) are encryption tiles (groups 0-2), [E, ntiles) decryption
-// tiles, with E = tile_end of group 2.  Every warp starts on a fixed tile,
-// then takes tiles from the direction's own counter until it runs dry,
-// independently of the other warps, so their global-memory latencies overlap.
-// The CTA meets at a barrier only to swap its shared-memory tables from the
-// encryption to the decryption set, once.
+// Units [0, E) are encryption units (groups 0-2), [E, ntiles << split) decryption
+// units.  The first enc_ctas CTAs begin with the encryption units, the others with
+// the decryption units (their numbers follow the lookups of each direction), so
+// both directions run at once and a CTA fills its tables once; one whose direction
+// has run dry swaps its tables and helps with the other, at one barrier.  Every
+// warp starts on a fixed unit of its CTA's direction (interleaved over the CTAs,
+// so a small batch spreads over the SMs), then takes units from the direction's
+// counter, independently of the other warps, so their global-memory latencies
+// overlap.  Without a counter (no direction has more units than warps) that is all.
 template <int BPT>
 __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const BatchArgs a) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -204,40 +244,46 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
             for (int k = 0; k < 8; ++k) sts(gaddr + 32u * i + 4u * k, w[k]);
         }
     }
-    __syncthreads();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t L0 = A | (lane << 2);
     const uint32_t L1 = L0 | 128u;
     const uint32_t kslot = kslots + 256u * (threadIdx.x >> 5);
-    const uint32_t enc_end = lds(gaddr + 32u * 2 + 4u);  // tile_end of group 2
-    int cur_dir = -1;
-    for (int dir = 0; dir < 2; ++dir) {
-        const uint32_t t_begin = dir ? enc_end : 0u;
-        const uint32_t t_end = dir ? a.ntiles : enc_end;
-        if (t_begin >= t_end) continue;  // same for the whole CTA
-        if (dir != cur_dir) {
-            __syncthreads();  // every warp has left the other direction's tiles
+    const uint32_t warps = blockDim.x >> 5;
+    const int first_dir = blockIdx.x < a.enc_ctas ? 0 : 1;
+    fill_tables(A, first_dir != 0);
+    __syncthreads();
+    const uint32_t enc_end = lds(gaddr + 32u * 2 + 4u) << a.split;  // tile_end of group 2
+    for (int phase = 0; phase < 2; ++phase) {
+        const int dir = phase ? first_dir ^ 1 : first_dir;
+        const uint32_t u_begin = dir ? enc_end : 0u;
+        const uint32_t count = (dir ? a.ntiles << a.split : enc_end) - u_begin;
+        const uint32_t ctas = dir ? gridDim.x - a.enc_ctas : a.enc_ctas;  // CTAs that begin with this direction
+        uint32_t u;
+        if (phase == 0) {
+            u = (threadIdx.x >> 5) * ctas + (dir ? blockIdx.x - a.enc_ctas : blockIdx.x);
+        } else {
+            if (!a.counter) return;
+            uint32_t left = 0;
+            if (threadIdx.x == 0) left = *(volatile unsigned*)(a.counter + dir) + ctas * warps < count;
+            if (!__syncthreads_or((int)left)) return;  // (every warp has left the other direction's units)
             fill_tables(A, dir != 0);
             __syncthreads();
-            cur_dir = dir;
+            u = 0;
+            if (lane == 0) u = atomicAdd(a.counter + dir, 1u) + ctas * warps;
+            u = __shfl_sync(0xffffffffu, u, 0);
         }
-        // Every warp's first tile is fixed (interleaved over the CTAs, so a
-        // small batch spreads over the SMs); later ones come from the
-        // direction's counter, offset by the number of fixed tiles.
-        const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
-        uint32_t t = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-        while (t < t_end - t_begin) {
-            uint32_t nxt = 0;
-            if (lane == 0) nxt = atomicAdd(a.counter + dir, 1u) + nwarps;  // consumed after this tile
-            t += t_begin;
+        while (u < count) {
+            uint32_t nxt = count;
+            if (a.counter && lane == 0) nxt = atomicAdd(a.counter + dir, 1u) + ctas * warps;  // consumed after this unit
+            const uint32_t t = (u + u_begin) >> a.split;
             int g = 0;
             while (g < kGroups - 1 && t >= lds(gaddr + 32u * g + 4u)) ++g;  // tile_end of group g
             const GroupDev G = load_group(gaddr, g);
             if (dir)
-                batch_warp_tile<true, BPT>(a, G, t, lane, L0, L1, kslot);
+                batch_warp_unit<true, BPT>(a, G, u + u_begin, lane, L0, L1, kslot);
             else
-                batch_warp_tile<false, BPT>(a, G, t, lane, L0, L1, kslot);
-            t = __shfl_sync(0xffffffffu, nxt, 0);
+                batch_warp_unit<false, BPT>(a, G, u + u_begin, lane, L0, L1, kslot);
+            u = __shfl_sync(0xffffffffu, nxt, 0);
         }
     }
 }
@@ -329,7 +375,8 @@ struct aes_batch_plan {
     HostPlan host;
     uint8_t* dev_buf;
     size_t dev_bytes;
-    BatchArgs args;  // device pointers filled in; in/out set per launch
+    BatchArgs args;  // device pointers and schedule filled in; in/out set per launch
+    uint32_t grid;
     cudaGraphExec_t graph_exec;
     cudaGraph_t graph;
     cudaGraphNode_t kernel_node;
@@ -395,23 +442,81 @@ static int batch_smem(BatchKernel fn, int* smem) {
     return AES_OK;
 }
 
-static unsigned batch_grid(uint32_t ntiles) {
-    DeviceInfo info;
-    if (current_device_info(&info)) return 1;
-    return (unsigned)std::min<uint64_t>(ntiles, (uint64_t)info.sms);
+// A tile is cut into the units that warps take, down to one pass of a warp,
+// until every warp has kUnitsPerWarp of them: a batch of few tiles spreads over
+// all warps, a large one keeps whole tiles (fewer unit starts).
+constexpr uint64_t kUnitsPerWarp = 4;
+
+// Up to this many blocks the two directions run side by side on CTAs of their
+// own (one table fill, one tail); above it every CTA begins with the encryption
+// tiles.  Side by side against one after the other: 50.7 / 66.1 us at 27 MB, 136.6 /
+// 150.3 at 85 MB, 400 / 408 at 291 MB, but 4,350 / 4,329 at 3.4 GB (512 x 8), where the
+// one fill and tail saved weigh less than what two streams of tiles cost.
+constexpr uint64_t kSideBySideBlocks = 1ull << 26;
+
+BatchSchedule schedule_batch(const HostPlan& H, int threads, int bpt, int sms) {
+    BatchSchedule s{};
+    const uint64_t warps = (uint64_t)threads / 32;
+    const uint32_t pass = 32u * (uint32_t)bpt;
+    while (((uint64_t)H.ntiles << s.split) < kUnitsPerWarp * warps * (uint64_t)sms &&
+           (H.tile_blocks >> s.split) % (2u * pass) == 0)
+        ++s.split;
+    const uint64_t units = (uint64_t)H.ntiles << s.split;
+    s.grid = (uint32_t)std::min<uint64_t>(units, (uint64_t)sms);
+    // CTAs to each direction by its lookups (16 per block and round).
+    uint64_t work[2] = {0, 0};
+    for (const GroupDev& G : H.groups) work[G.dir] += G.blocks * (uint64_t)G.nr;
+    const uint64_t enc_units = (uint64_t)H.groups[kGroups / 2 - 1].tile_end << s.split;
+    if (work[0] && work[1] && H.total_blocks <= kSideBySideBlocks) {
+        const double share = (double)work[0] / ((double)work[0] + (double)work[1]);
+        s.enc_ctas = (uint32_t)(share * s.grid + 0.5);
+        s.enc_ctas = std::min(std::max(s.enc_ctas, 1u), s.grid - 1u);
+    } else {
+        s.enc_ctas = work[0] ? s.grid : 0u;
+    }
+    s.counted = enc_units > s.enc_ctas * warps || units - enc_units > (s.grid - s.enc_ctas) * warps;
+    return s;
 }
 
-int launch_batch_kernel(const BatchArgs& a, int threads, int bpt, cudaStream_t stream) {
+static BatchSchedule current_schedule(const HostPlan& H, int threads, int bpt) {
+    DeviceInfo info;
+    return schedule_batch(H, threads, bpt, current_device_info(&info) ? 1 : info.sms);
+}
+
+int launch_batch_kernel(const HostPlan& H, BatchArgs a, int threads, int bpt, cudaStream_t stream) {
     BatchKernel fn = pick_batch(bpt);
     if (!fn) return fail(AES_ERR_ARG, "blocks_per_thread %d: need 1, 2, 4 or 8", bpt);
     if (bpt == 8 && threads > 512) return fail(AES_ERR_ARG, "8 blocks per thread need threads <= 512");
     int smem = 0;
     int rc = batch_smem(fn, &smem);
     if (rc) return rc;
-    fn<<<batch_grid(a.ntiles), threads, smem, stream>>>(a);
+    const BatchSchedule sch = current_schedule(H, threads, bpt);
+    a.split = sch.split;
+    a.enc_ctas = sch.enc_ctas;
+    if (!sch.counted) a.counter = nullptr;
+    fn<<<sch.grid, threads, smem, stream>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "batch kernel launch: %s", cudaGetErrorString(e));
     return AES_OK;
+}
+
+// Tile size and launch shape of a call that plans for one launch (kept plans
+// take theirs from the caller).
+constexpr uint32_t kOneShotTileMax = 2048;
+
+struct OneShot {
+    uint32_t tile_blocks;
+    int threads, bpt;
+};
+
+// 1024 x 2 at every size: 14.6 us for 2,000 messages of 16 B - 16 KiB (4.7 MB) against
+// 19.2 with 1024 x 1 and 16.6 with 512 x 8; 50.6 / 53.6 / 50.9 at 27 MB.  Above 2^23
+// blocks tiles of 512 would only lengthen the upload.
+static OneShot one_shot_shape(const aes_msg_desc* d, size_t nmsg) {
+    uint64_t total = 0;
+    for (size_t i = 0; d && i < nmsg; ++i) total += std::min<uint64_t>(d[i].nblocks, 1ull << 32);
+    if (total <= 1u << 23) return OneShot{512, 1024, 2};
+    return OneShot{kOneShotTileMax, 1024, 2};
 }
 
 }  // namespace gbaes
@@ -488,6 +593,13 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
     a.ntiles = H.ntiles;
     a.tile_blocks = H.tile_blocks;
     memcpy(a.groups, H.groups, sizeof a.groups);
+    if (H.ntiles) {
+        const BatchSchedule sch = current_schedule(H, P->threads, P->bpt);
+        a.split = sch.split;
+        a.enc_ctas = sch.enc_ctas;
+        if (!sch.counted) a.counter = nullptr;
+        P->grid = sch.grid;
+    }
     P->magic = kPlanMagic;
     return P;
 }
@@ -503,9 +615,10 @@ int aes_batch_plan_launch(aes_batch_plan* P, const void* in_base, size_t in_byte
     rc = batch_smem(fn, &smem);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(a.counter, 0, 2 * sizeof(unsigned), s);
+    cudaError_t e = cudaSuccess;
+    if (a.counter) e = cudaMemsetAsync(a.counter, 0, 2 * sizeof(unsigned), s);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "resetting the tile counter: %s", cudaGetErrorString(e));
-    fn<<<batch_grid(P->host.ntiles), P->threads, smem, s>>>(a);
+    fn<<<P->grid, P->threads, smem, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "batch kernel launch: %s", cudaGetErrorString(e));
     return AES_OK;
@@ -530,8 +643,8 @@ int aes_batch_plan_launch_graph(aes_batch_plan* P, const void* in_base, size_t i
         }
         e = cudaStreamBeginCapture(P->capture_stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            cudaMemsetAsync(a.counter, 0, 2 * sizeof(unsigned), P->capture_stream);
-            fn<<<batch_grid(P->host.ntiles), P->threads, smem, P->capture_stream>>>(a);
+            if (a.counter) cudaMemsetAsync(a.counter, 0, 2 * sizeof(unsigned), P->capture_stream);
+            fn<<<P->grid, P->threads, smem, P->capture_stream>>>(a);
             e = cudaStreamEndCapture(P->capture_stream, &P->graph);
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&P->graph_exec, P->graph, 0);
@@ -555,7 +668,7 @@ int aes_batch_plan_launch_graph(aes_batch_plan* P, const void* in_base, size_t i
         cudaKernelNodeParams kp;
         memset(&kp, 0, sizeof kp);
         kp.func = (void*)fn;
-        kp.gridDim = dim3(batch_grid(P->host.ntiles));
+        kp.gridDim = dim3(P->grid);
         kp.blockDim = dim3(P->threads);
         kp.sharedMemBytes = smem;
         kp.kernelParams = params;
@@ -595,7 +708,8 @@ int aes_ecb_batch(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* c
                     "aes_ecb_batch uploads from host memory freed on return and cannot be captured; "
                     "use aes_batch_plan_launch_graph");
     HostPlan H;
-    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, 2048, true, &H);
+    const OneShot shape = one_shot_shape(msgs, nmsg);
+    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, true, &H);
     if (rc) return rc;
     if (H.ntiles == 0) return AES_OK;
     rc = check_bases(H, in_base, in_bytes, out_base, out_bytes);
@@ -631,18 +745,9 @@ int aes_ecb_batch(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* c
     a.ntiles = H.ntiles;
     a.tile_blocks = H.tile_blocks;
     memcpy(a.groups, H.groups, sizeof a.groups);
-    BatchKernel fn = pick_batch(2);
-    int smem = 0;
-    rc = batch_smem(fn, &smem);
-    if (rc) {
-        cudaFreeAsync(buf, s);
-        return rc;
-    }
-    fn<<<batch_grid(H.ntiles), 1024, smem, s>>>(a);
-    e = cudaGetLastError();
+    rc = launch_batch_kernel(H, a, shape.threads, shape.bpt, s);
     cudaFreeAsync(buf, s);
-    if (e != cudaSuccess) return fail(AES_ERR_CUDA, "batch kernel launch: %s", cudaGetErrorString(e));
-    return AES_OK;
+    return rc;
 }
 
 int aes_batch_tiles(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx, int tile_blocks,
@@ -710,15 +815,22 @@ extern "C" {
 int aes_ecb_batch_noalloc(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx,
                           const void* in_base, size_t in_bytes, void* out_base, size_t out_bytes, void* stream) {
     HostPlan H;
-    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, 2048, true, &H);
-    if (rc) return rc;
+    OneShot shape = one_shot_shape(msgs, nmsg);
+    size_t off_keys = 256, off_msgs = 0, off_tiles = 0, bytes = 0;  // [0, 256): tile counter, uploaded as zero
+    int rc = AES_OK;
+    for (;;) {
+        rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, true, &H);
+        if (rc) return rc;
+        off_msgs = off_keys + align256(H.keys.size() * 4);
+        off_tiles = off_msgs + align256(H.msgs.size() * sizeof(MsgDev));
+        bytes = off_tiles + align256(H.tile_msg.size() * 4 + 4);
+        if (bytes <= kNoAllocScratchBytes || shape.tile_blocks == kOneShotTileMax) break;
+        shape.tile_blocks = kOneShotTileMax;  // the smallest tables
+        H = HostPlan();
+    }
     if (H.ntiles == 0) return AES_OK;
     rc = check_bases(H, in_base, in_bytes, out_base, out_bytes);
     if (rc) return rc;
-    const size_t off_keys = 256;  // [0, 256): tile counter, uploaded as zero
-    const size_t off_msgs = off_keys + align256(H.keys.size() * 4);
-    const size_t off_tiles = off_msgs + align256(H.msgs.size() * sizeof(MsgDev));
-    const size_t bytes = off_tiles + align256(H.tile_msg.size() * 4 + 4);
     if (bytes > kNoAllocScratchBytes)
         return fail(AES_ERR_ARG,
                     "batch needs %zu bytes of tables (keys: 512 B per context; 32 B per message; 4 B per tile), "
@@ -729,10 +841,6 @@ int aes_ecb_batch_noalloc(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* 
     if (rc) return rc;
     int* status = nullptr;
     rc = device_status_word(&status);
-    if (rc) return rc;
-    BatchKernel fn = pick_batch(2);
-    int smem = 0;
-    rc = batch_smem(fn, &smem);
     if (rc) return rc;
     std::vector<uint8_t> img(bytes, 0);  // host staging only; the counter word stays zero
     memcpy(img.data() + off_keys, H.keys.data(), H.keys.size() * 4);
@@ -755,10 +863,7 @@ int aes_ecb_batch_noalloc(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* 
     a.ntiles = H.ntiles;
     a.tile_blocks = H.tile_blocks;
     memcpy(a.groups, H.groups, sizeof a.groups);
-    fn<<<batch_grid(H.ntiles), 1024, smem, s>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(AES_ERR_CUDA, "batch kernel launch: %s", cudaGetErrorString(e));
-    return AES_OK;
+    return launch_batch_kernel(H, a, shape.threads, shape.bpt, s);
 }
 
 }  // extern "C"

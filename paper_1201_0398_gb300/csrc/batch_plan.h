@@ -36,10 +36,12 @@ struct BatchArgs {
     const MsgDev* msgs;
     const uint4* keys;  // kSlotWords / 4 uint4 per slot
     const uint32_t* tile_msg;
-    unsigned* counter;
+    unsigned* counter;  // two words (zero at the launch), or nullptr: no direction has more units than warps
     int* status;
     uint32_t ntiles;
     uint32_t tile_blocks;
+    uint32_t split;     // a warp takes 1 / 2^split of a tile at a time
+    uint32_t enc_ctas;  // CTAs that begin with the encryption tiles
     GroupDev groups[kGroups];
 };
 
@@ -59,8 +61,18 @@ struct HostPlan {
 int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx, uint32_t tile_blocks,
                     bool with_keys, HostPlan* P);
 
-// Launches the batched kernel (one CTA per SM at most; ntiles > 0).
-int launch_batch_kernel(const BatchArgs& a, int threads, int bpt, cudaStream_t stream);
+// How one batched launch shares its tiles among the GPU's warps (BatchArgs::split, enc_ctas).
+struct BatchSchedule {
+    uint32_t split;
+    uint32_t enc_ctas;
+    uint32_t grid;
+    bool counted;  // some warps take more than one unit: the launch needs its counter, zeroed
+};
+BatchSchedule schedule_batch(const HostPlan& H, int threads, int bpt, int sms);
+
+// Launches the batched kernel (one CTA per SM at most; ntiles > 0): fills in a.split, a.enc_ctas and, where the
+// schedule needs none, clears a.counter.
+int launch_batch_kernel(const HostPlan& H, BatchArgs a, int threads, int bpt, cudaStream_t stream);
 
 int device_status_word(int** p);  // ecb_table.cu
 

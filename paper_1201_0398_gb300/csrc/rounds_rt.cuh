@@ -67,12 +67,16 @@ struct OneGlobalKey {
     __device__ __forceinline__ uint4 get(int r, int) const { return __ldg(p + r); }
 };
 
-// A schedule in global memory per state (states of different messages).
-template <int BPT>
+// A schedule in global memory per state (states of different messages): slots of
+// kSlotWords words from `keys` (32-bit slot numbers, half a pointer's registers).
+template <int BPT, int SLOT_UINT4>
 struct StateKeys {
     static constexpr bool kPerState = true;
-    const uint4* const (&p)[BPT];
-    __device__ __forceinline__ uint4 get(int r, int b) const { return __ldg(p[b] + r); }
+    const uint4* keys;
+    const uint32_t (&slot)[BPT];
+    __device__ __forceinline__ uint4 get(int r, int b) const {
+        return __ldg(keys + (uint64_t)slot[b] * SLOT_UINT4 + r);
+    }
 };
 
 }  // namespace gbaes

@@ -737,7 +737,7 @@ static int launch_slot(aes_server* S, Slot& slot) {
     a.ntiles = H.ntiles;
     a.tile_blocks = H.tile_blocks;
     memcpy(a.groups, H.groups, sizeof a.groups);
-    rc = launch_batch_kernel(a, S->cfg.threads, S->cfg.blocks_per_thread, slot.stream);
+    rc = launch_batch_kernel(H, a, S->cfg.threads, S->cfg.blocks_per_thread, slot.stream);
     if (rc) return rc;
     e = cudaEventRecord(slot.done, slot.stream);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "batch event: %s", cudaGetErrorString(e));

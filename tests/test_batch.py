@@ -134,6 +134,44 @@ def test_batch_vs_oracle_and_single_kernel(gbaes, threads, bpt):
     assert gbaes.device_status() == 0
 
 
+# Message lengths in blocks, at the edges of how a warp finds each block's message: it looks at the starts of
+# the next 32 messages at once, takes 32 blocks per pass and state, and units of a few hundred blocks.
+EDGES = {
+    "one": [1],
+    "ones": [1] * 700,  # a window of starts is used up every 32 blocks
+    "ones_then_long": [1] * 31 + [2000] + [1] * 33 + [64] + [1] * 64 + [513],
+    "whole_passes": [32] * 40 + [64] * 20 + [256] * 3,  # boundaries at the first block of a pass
+    "off_by_one": [31, 33, 32, 1, 63, 65, 31, 1, 127, 129, 255, 257, 511, 513, 1, 2047, 2049],
+    "long": [70_001],
+}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("lengths", EDGES)
+@pytest.mark.parametrize("threads,bpt", [(64, 1), (1024, 2), (1024, 4), (512, 8)])
+@pytest.mark.parametrize("directions", ["enc", "dec", "both"])
+def test_batch_message_boundaries(gbaes, lengths, threads, bpt, directions):
+    rng = np.random.default_rng(len(lengths))
+    nblocks = np.array(EDGES[lengths], np.int64)
+    n = len(nblocks)
+    bits = np.array([128] * n) if lengths == "long" else rng.choice([128, 128, 256], n)
+    keys = [rng.integers(0, 256, b // 8, dtype=np.uint8).tobytes() for b in bits]
+    ks = [gbaes.Key(k) for k in keys]
+    decrypt = {"enc": np.zeros(n, int), "dec": np.ones(n, int), "both": np.arange(n) % 2}[directions]
+    off = (np.cumsum(nblocks) - nblocks) * 16
+    data = rng.integers(0, 256, 16 * int(nblocks.sum()), dtype=np.uint8)
+    d = gbaes.make_descs(off, off, nblocks, np.arange(n), decrypt)
+    want = oracle_batch(data, keys, bits, nblocks, np.arange(n), decrypt, off, off, data.size)
+    x = torch.from_numpy(data).cuda()
+    plan = gbaes.BatchPlan(d, ks, threads, bpt)
+    for launch in (lambda y: plan.launch(x, y), lambda y: plan.launch(x, y, graph=True),
+                   lambda y: plan.launch(x, y, graph=True), lambda y: gbaes.ecb_batch(d, ks, x, y)):
+        y = torch.zeros_like(x)
+        launch(y)
+        assert np.array_equal(host(y), want)
+    assert gbaes.device_status() == 0
+
+
 @pytest.mark.gpu
 def test_batch_graph_rebase_one_shot_and_in_place(gbaes):
     rng = np.random.default_rng(42)
