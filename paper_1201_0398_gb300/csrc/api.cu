@@ -329,6 +329,12 @@ static int run_block_op(const aes_ctx* ctx, Mode mode, const void* in, void* out
         a.first = first;
     }
     if (mode == kCbcDec) memcpy(a.iv, iv, 16);
+    if (mode == kCtr) {
+        DeviceInfo info;
+        rc = current_device_info(&info);
+        if (rc) return rc;
+        if (nblocks >= ctr_min_blocks(info.sms)) return launch_ctr(a, ctx->nr, (cudaStream_t)stream);
+    }
     if (kernel == AES_KERNEL_BITSLICED) {
         if (mode != kEnc && mode != kDec) return fail(AES_ERR_ARG, "the bitsliced kernel implements ECB only");
         return launch_bitsliced(a, ctx->enc_rk, ctx->nr, mode, threads, (cudaStream_t)stream);

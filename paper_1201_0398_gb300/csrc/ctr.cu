@@ -1,0 +1,167 @@
+// CTR mode on long inputs: the first two rounds shared between blocks.
+//
+// Section 3's CTR listing enciphers a counter per block, and counters that follow
+// one another differ in one or two bytes.  Take the blocks whose counters agree in
+// the upper 14 bytes, and call the two lowest bytes y and x.  After round 1 of
+// Eq. 1 column 0 depends on x alone, another column on y alone (1 for the
+// big-endian counter, 3 for the little-endian one) and two on neither; round 2
+// XORs one lookup of each column into every word, so the state after it is
+//     F(x, y) = A(x) ^ B(y) = F(x, y0) ^ F(0, y0) ^ F(0, y).
+// (Sharing the first rounds of neighbouring counters is Bernstein and Schwabe's
+// "counter-mode caching", New AES Software Speed Records, 2008; splitting round 2
+// in two parts, each common to many blocks, spares all 32 lookups of both rounds.)
+//
+// Rows of 256 counters share y.  A warp takes 32 neighbouring x of consecutive
+// rows: its lanes keep F(x, y0) ^ F(0, y0) in four registers while the upper 14
+// bytes last (2^16 counters), and F(0, y) of the next 32 rows -- the same for all
+// lanes -- in shared memory, one 16-byte broadcast load per row in place of 32
+// lookups.  Both come from two ordinary rounds, 32 lookups per lane each.
+//
+// Bound: the shared-memory lookups of the remaining Nr - 2 rounds (16 per block and
+// round, 32 lanes per clock and SM) and the L1 cycles of the global loads and
+// stores (about 16 per 32 blocks): 1 GiB of AES-128 takes 147 of the 128 + 16
+// cycles per 32 blocks, where the table kernel's ten rounds take 177.  Measured,
+// before and after: 1 GiB 908 -> 1,117 GB/s (AES-256 667 -> 771; 1,104 / 766 where the
+// input's first counter is odd, so that a warp's 512 bytes straddle five lines),
+// 256 MiB 894 -> 1,079 (658 -> 752), 16 MiB 788 -> 887 (598 -> 649).
+#include "block_io.cuh"
+#include "rounds_dp4a.cuh"
+
+namespace gbaes {
+
+constexpr int kCtrThreads = 512;  // 8 warps span a row's 256 counters; 2 row ranges per CTA
+constexpr int kCtrHalves = kCtrThreads / 256;
+constexpr int kCtrRows = 4;         // rows a warp enciphers at a time
+constexpr uint32_t kCtrSlots = 32;  // rows whose F(0, y) a warp keeps
+constexpr uint32_t kCtrSmem = dp::kEncBytes + (kCtrThreads / 32) * kCtrSlots * 16u;
+
+// Rows row .. row + ROWS - 1 of this warp: v = 256 row + x is a block's counter
+// less the (2^16-aligned) counter base, and v - a.first its place in the input;
+// places outside the input (before its first counter, past its last) compute and
+// store nothing.
+template <int NR, int ROWS>
+__device__ __forceinline__ void ctr_rows(const EcbArgs& a, uint64_t row, uint32_t x, const uint32_t (&ax)[4],
+                                         uint32_t slots, uint32_t L) {
+    uint32_t s[ROWS][4];
+    uint4 data[ROWS];
+    const uint64_t i0 = (row << 8) + x - a.first;
+#pragma unroll
+    for (int b = 0; b < ROWS; ++b) {
+        const uint64_t i = i0 + 256u * b;
+        data[b] = i < a.nblocks ? ld_stream(a.in + i) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int b = 0; b < ROWS; ++b) {
+        uint4 f;
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(f.x), "=r"(f.y), "=r"(f.z), "=r"(f.w)
+                     : "r"(slots + 16u * (((uint32_t)row + b) % kCtrSlots)));
+        s[b][0] = ax[0] ^ f.x;
+        s[b][1] = ax[1] ^ f.y;
+        s[b][2] = ax[2] ^ f.z;
+        s[b][3] = ax[3] ^ f.w;
+    }
+    dp::rounds_from<NR, false, 3, ROWS>(s, ParamKeys{a.rk}, L);
+#pragma unroll
+    for (int b = 0; b < ROWS; ++b) {
+        const uint64_t i = i0 + 256u * b;
+        if (i < a.nblocks) store_block<kCtr>(a, i, s[b], data[b]);
+    }
+}
+
+// The states after two rounds of the counters v[i] past the base.
+template <int N>
+__device__ __forceinline__ void two_rounds(const EcbArgs& a, const uint64_t (&v)[N], uint32_t L, uint32_t (&s)[N][4]) {
+    const ParamKeys ks{a.rk};
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        counter_words(a, v[i], s[i]);
+        const uint4 k = ks.get(0);
+        s[i][0] ^= k.x;
+        s[i][1] ^= k.y;
+        s[i][2] ^= k.z;
+        s[i][3] ^= k.w;
+    }
+#pragma unroll
+    for (int r = 1; r <= 2; ++r)
+#pragma unroll
+        for (int i = 0; i < N; ++i) dp::round_inner<false>(s[i], L, ks.get(r));
+}
+
+// a.ctr_hi, a.ctr_lo: the counter base, its low 16 bits 0; a.first: the first
+// block's counter less the base (below 2^16).
+template <int NR>
+__global__ void __launch_bounds__(kCtrThreads, 1) ctr_kernel(const __grid_constant__ EcbArgs a) {
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    const uint32_t A = smem_base(smem_raw);
+    dp::fill_tables<kCtrThreads, false>(A);
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t L = A + 4u * lane;
+    const uint32_t slots = A + dp::kEncBytes + (threadIdx.x >> 5) * kCtrSlots * 16u;
+    const uint32_t x = threadIdx.x & 255u;
+    // Rows with blocks of the input, shared out evenly over the row ranges of all CTAs.
+    const uint64_t row0 = a.first >> 8;
+    const uint64_t rows = ((a.first + a.nblocks - 1) >> 8) - row0 + 1;
+    const uint64_t range = (uint64_t)blockIdx.x * kCtrHalves + (threadIdx.x >> 8);
+    const uint64_t ranges = (uint64_t)gridDim.x * kCtrHalves;
+    uint64_t row = row0 + rows * range / ranges;
+    const uint64_t end = row0 + rows * (range + 1) / ranges;
+    uint64_t high = ~0ull;  // row / 256 that ax belongs to
+    uint32_t ax[4] = {0, 0, 0, 0};
+    while (row < end) {
+        const uint64_t slot_row = row & ~(uint64_t)(kCtrSlots - 1);
+        uint32_t f[4];
+        if (row >> 8 != high) {
+            high = row >> 8;
+            uint32_t t[2][4];
+            two_rounds<2>(a, {(slot_row + lane) << 8, (slot_row << 8) + x}, L, t);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                f[w] = t[0][w];
+                ax[w] = t[1][w] ^ __shfl_sync(0xffffffffu, f[w], 0);
+            }
+        } else {
+            uint32_t t[1][4];
+            two_rounds<1>(a, {(slot_row + lane) << 8}, L, t);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) f[w] = t[0][w];
+        }
+        __syncwarp();  // every lane is done with the slots' previous rows
+        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(slots + 16u * lane), "r"(f[0]), "r"(f[1]),
+                     "r"(f[2]), "r"(f[3])
+                     : "memory");
+        __syncwarp();
+        const uint64_t stop = slot_row + kCtrSlots < end ? slot_row + kCtrSlots : end;
+        for (; row + kCtrRows <= stop; row += kCtrRows) ctr_rows<NR, kCtrRows>(a, row, x, ax, slots, L);
+        for (; row < stop; ++row) ctr_rows<NR, 1>(a, row, x, ax, slots, L);
+    }
+}
+
+// Shortest input that takes this kernel: five rows for every row range.  With
+// fewer the two rounds ahead of a range's first row and the uneven last rows cost
+// more than the rounds spared: 311,296 blocks (four rows) 8.28 us in the table kernel,
+// 8.47 here (AES-256 10.34 / 10.75), 400,000 blocks 10.57 / 9.85 (13.48 / 12.76).
+uint64_t ctr_min_blocks(int sms) { return (uint64_t)sms * kCtrHalves * 256u * 5u; }
+
+int launch_ctr(EcbArgs a, int nr, cudaStream_t stream) {
+    DeviceInfo info;
+    int rc = current_device_info(&info);
+    if (rc) return rc;
+    using Fn = void (*)(const EcbArgs);
+    const Fn fn = nr == 10 ? ctr_kernel<10> : nr == 12 ? ctr_kernel<12> : nr == 14 ? ctr_kernel<14> : nullptr;
+    if (!fn) return fail(AES_ERR_ARG, "no CTR kernel for nr=%d", nr);
+    rc = set_max_dynamic_smem((const void*)fn, kCtrSmem);
+    if (rc) return rc;
+    // The first counter, split into a base with 16 zero low bits and the rest.
+    const uint64_t lo = a.ctr_lo + a.first;
+    if (lo < a.ctr_lo) ++a.ctr_hi;
+    a.ctr_lo = lo & ~0xffffull;
+    a.first = lo & 0xffffull;
+    fn<<<info.sms, kCtrThreads, kCtrSmem, stream>>>(a);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return fail(AES_ERR_CUDA, "CTR kernel launch: %s", cudaGetErrorString(e));
+    return AES_OK;
+}
+
+}  // namespace gbaes

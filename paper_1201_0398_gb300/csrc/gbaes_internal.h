@@ -83,6 +83,10 @@ uint64_t compact_limit_blocks(int sms);
 // and bpt shape the replicated kernel only.
 int launch_table(const EcbArgs& a, int nr, Mode mode, int threads, int bpt, int variant, cudaStream_t stream);
 
+// CTR on inputs of at least ctr_min_blocks blocks (ctr.cu); a.first is any 64-bit index.
+uint64_t ctr_min_blocks(int sms);
+int launch_ctr(EcbArgs a, int nr, cudaStream_t stream);
+
 // Launches the bitsliced kernel (ecb_bitsliced.cu), ECB only.
 int launch_bitsliced(const EcbArgs& a, const uint32_t* enc_rk, int nr, Mode mode, int threads, cudaStream_t stream);
 

@@ -157,6 +157,36 @@ def test_ctr_vs_oracle(gbaes, bits):
 
 
 @pytest.mark.parametrize("bits", BITS)
+@pytest.mark.parametrize("kind", ("CTR_BE128", "CTR_LE32_CARRY"))
+def test_ctr_long_inputs_share_their_first_rounds(gbaes, bits, kind):
+    """Inputs from the length at which rows of 256 counters share the first two
+    rounds (one block below it, at it, and with ragged last rows), from first
+    counters at the edges of a row, of the 2^16 counters that agree in their
+    upper bytes, of a 64-bit half and of 2^128, and with a block index: as the
+    oracle computes them from the counter that comes out, and in place."""
+    rng = np.random.default_rng(bits)
+    key = rng.integers(0, 256, bits // 8, dtype=np.uint8).tobytes()
+    k = gbaes.Key(key)
+    least = sms() * 2 * 256 * 5
+    order = "big" if kind == "CTR_BE128" else "little"
+    nonce = int.from_bytes(rng.integers(0, 256, 16, dtype=np.uint8).tobytes(), "big") & ~((1 << 64) - 1)
+    firsts = (nonce, nonce | 0xFF, nonce | 0x100, nonce | 0xFFFF, nonce | 0x12FFE1, nonce | ((1 << 64) - 70_000),
+              (1 << 128) - 1)
+    data = rng.integers(0, 256, 16 * (least + 9001), dtype=np.uint8)
+    x = dev(data)
+    for j, first in enumerate(firsts):
+        n = least + (0, 1, -1, 255, 9001, 31, 4096)[j]
+        index = (0, 3, 1 << 40, 65_537, 0, (1 << 64) - n - 1, 12_345)[j]
+        iv = ((first - index) % (1 << 128)).to_bytes(16, order)
+        got = gbaes.ctr_xcrypt(k, iv, x[:16 * n], kind=getattr(gbaes, kind), first_block=index)
+        want = oracle.ctr(key, bits, first.to_bytes(16, order), data[:16 * n], getattr(oracle, kind))
+        assert np.array_equal(host(got), want), (hex(first), n, index)
+    gbaes.ctr_xcrypt(k, iv, x[:16 * n], out=x[:16 * n], kind=getattr(gbaes, kind), first_block=index)
+    assert np.array_equal(host(x[:16 * n]), want) and np.array_equal(host(x[16 * n:]), data[16 * n:])
+    assert gbaes.device_status() == 0
+
+
+@pytest.mark.parametrize("bits", BITS)
 def test_cbc_decrypt_vs_oracle(gbaes, bits):
     rng = np.random.default_rng(700 + bits)
     key = rng.integers(0, 256, bits // 8, dtype=np.uint8).tobytes()
