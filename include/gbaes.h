@@ -153,16 +153,15 @@ typedef struct aes_batch_plan aes_batch_plan;
 aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx,
                                       int threads, int blocks_per_thread);
 
-/* Launches a plan on `stream`: resets the plan's tile counters (a batch with no
- * more parts than warps needs none), then one persistent kernel (one CTA per SM; its warps take tiles independently).  in_base/out_base: device buffers of
+/* Launches a plan on `stream`: one persistent kernel (one CTA per SM; its warps take tiles independently).  in_base/out_base: device buffers of
  * in_bytes/out_bytes bytes that must cover every message (AES_ERR_ARG).  Two
  * launches of the same plan must not run concurrently (they share its tile
  * counter); stream-ordered repeats are fine. */
 int aes_batch_plan_launch(aes_batch_plan* plan, const void* in_base, size_t in_bytes, void* out_base,
                           size_t out_bytes, void* stream);
 
-/* Same as aes_batch_plan_launch through a CUDA graph captured on first use
- * (counter reset + kernel) and replayed afterwards; new base pointers update
+/* Same as aes_batch_plan_launch through a CUDA graph of the kernel, captured on
+ * first use and replayed afterwards; new base pointers update
  * the captured kernel's arguments.  Same concurrency rule. */
 int aes_batch_plan_launch_graph(aes_batch_plan* plan, const void* in_base, size_t in_bytes, void* out_base,
                                 size_t out_bytes, void* stream);

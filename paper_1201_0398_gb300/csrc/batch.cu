@@ -34,6 +34,7 @@
 
 #include "aes_rounds.cuh"
 #include "batch_plan.h"
+#include "launch.cuh"
 #include "rounds_rt.cuh"
 
 namespace gbaes {
@@ -223,6 +224,7 @@ __device__ __forceinline__ GroupDev load_group(uint32_t gaddr, int g) {
 // overlap.  Without a counter (no direction has more units than warps) that is all.
 template <int BPT>
 __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const BatchArgs a) {
+    pdl_trigger();
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t base = smem_base(smem_raw);
     const uint32_t A = table_base(base);
@@ -252,6 +254,7 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
     const int first_dir = blockIdx.x < a.enc_ctas ? 0 : 1;
     fill_tables(A, first_dir != 0);
     __syncthreads();
+    pdl_wait();
     const uint32_t enc_end = lds(gaddr + 32u * 2 + 4u) << a.split;  // tile_end of group 2
     for (int phase = 0; phase < 2; ++phase) {
         const int dir = phase ? first_dir ^ 1 : first_dir;
@@ -262,10 +265,10 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
         if (phase == 0) {
             u = (threadIdx.x >> 5) * ctas + (dir ? blockIdx.x - a.enc_ctas : blockIdx.x);
         } else {
-            if (!a.counter) return;
+            if (!a.counter) return;  // (every direction's units were given out at the start)
             uint32_t left = 0;
             if (threadIdx.x == 0) left = *(volatile unsigned*)(a.counter + dir) + ctas * warps < count;
-            if (!__syncthreads_or((int)left)) return;  // (every warp has left the other direction's units)
+            if (!__syncthreads_or((int)left)) break;  // (every warp has left the other direction's units)
             fill_tables(A, dir != 0);
             __syncthreads();
             u = 0;
@@ -284,6 +287,17 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
             else
                 batch_warp_unit<false, BPT>(a, G, u + u_begin, lane, L0, L1, kslot);
             u = __shfl_sync(0xffffffffu, nxt, 0);
+        }
+    }
+    // The last CTA to get here leaves the counters at zero for the next launch of
+    // these tables (which waits for this one's end).
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(a.counter + kCtasDone, 1u) == gridDim.x - 1) {
+            a.counter[0] = 0;
+            a.counter[1] = 0;
+            a.counter[kCtasDone] = 0;
         }
     }
 }
@@ -494,8 +508,7 @@ int launch_batch_kernel(const HostPlan& H, BatchArgs a, int threads, int bpt, cu
     a.split = sch.split;
     a.enc_ctas = sch.enc_ctas;
     if (!sch.counted) a.counter = nullptr;
-    fn<<<sch.grid, threads, smem, stream>>>(a);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_overlapped(fn, sch.grid, (unsigned)threads, (size_t)smem, stream, a);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "batch kernel launch: %s", cudaGetErrorString(e));
     return AES_OK;
 }
@@ -614,12 +627,7 @@ int aes_batch_plan_launch(aes_batch_plan* P, const void* in_base, size_t in_byte
     int smem = 0;
     rc = batch_smem(fn, &smem);
     if (rc) return rc;
-    cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaSuccess;
-    if (a.counter) e = cudaMemsetAsync(a.counter, 0, 2 * sizeof(unsigned), s);
-    if (e != cudaSuccess) return fail(AES_ERR_CUDA, "resetting the tile counter: %s", cudaGetErrorString(e));
-    fn<<<P->grid, P->threads, smem, s>>>(a);
-    e = cudaGetLastError();
+    const cudaError_t e = launch_overlapped(fn, P->grid, (unsigned)P->threads, (size_t)smem, (cudaStream_t)stream, a);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "batch kernel launch: %s", cudaGetErrorString(e));
     return AES_OK;
 }
@@ -643,7 +651,6 @@ int aes_batch_plan_launch_graph(aes_batch_plan* P, const void* in_base, size_t i
         }
         e = cudaStreamBeginCapture(P->capture_stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            if (a.counter) cudaMemsetAsync(a.counter, 0, 2 * sizeof(unsigned), P->capture_stream);
             fn<<<P->grid, P->threads, smem, P->capture_stream>>>(a);
             e = cudaStreamEndCapture(P->capture_stream, &P->graph);
         }

@@ -28,6 +28,7 @@ struct GroupDev {
 };
 
 constexpr int kGroups = 6;
+constexpr int kCtasDone = 2;  // BatchArgs::counter[kCtasDone]
 constexpr int kSlotWords = 64;  // 60 used (Nr = 14), padded to 256 bytes
 
 struct BatchArgs {
@@ -36,7 +37,8 @@ struct BatchArgs {
     const MsgDev* msgs;
     const uint4* keys;  // kSlotWords / 4 uint4 per slot
     const uint32_t* tile_msg;
-    unsigned* counter;  // two words (zero at the launch), or nullptr: no direction has more units than warps
+    unsigned* counter;  // three words, zero at the launch and after it (units taken of each direction, CTAs done),
+                        // or nullptr: no direction has more units than warps
     int* status;
     uint32_t ntiles;
     uint32_t tile_blocks;

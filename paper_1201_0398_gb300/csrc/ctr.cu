@@ -25,6 +25,7 @@
 // input's first counter is odd, so that a warp's 512 bytes straddle five lines),
 // 256 MiB 894 -> 1,079 (658 -> 752), 16 MiB 788 -> 887 (598 -> 649).
 #include "block_io.cuh"
+#include "launch.cuh"
 #include "rounds_dp4a.cuh"
 
 namespace gbaes {
@@ -91,11 +92,13 @@ __device__ __forceinline__ void two_rounds(const EcbArgs& a, const uint64_t (&v)
 // a.ctr_hi, a.ctr_lo: the counter base, its low 16 bits 0; a.first: the first
 // block's counter less the base (below 2^16).
 template <int NR>
-__global__ void __launch_bounds__(kCtrThreads, 1) ctr_kernel(const __grid_constant__ EcbArgs a) {
+__global__ void __launch_bounds__(kCtrThreads, 1) ctr_kernel(const EcbArgs a) {
+    pdl_trigger();
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t A = smem_base(smem_raw);
     dp::fill_tables<kCtrThreads, false>(A);
     __syncthreads();
+    pdl_wait();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t L = A + 4u * lane;
     const uint32_t slots = A + dp::kEncBytes + (threadIdx.x >> 5) * kCtrSlots * 16u;
@@ -158,8 +161,7 @@ int launch_ctr(EcbArgs a, int nr, cudaStream_t stream) {
     if (lo < a.ctr_lo) ++a.ctr_hi;
     a.ctr_lo = lo & ~0xffffull;
     a.first = lo & 0xffffull;
-    fn<<<info.sms, kCtrThreads, kCtrSmem, stream>>>(a);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_overlapped(fn, (unsigned)info.sms, kCtrThreads, kCtrSmem, stream, a);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "CTR kernel launch: %s", cudaGetErrorString(e));
     return AES_OK;
 }

@@ -19,6 +19,7 @@
 #include <mutex>
 
 #include "bitsliced.h"
+#include "launch.cuh"
 #include "gbaes_internal.h"
 
 namespace gbaes {
@@ -46,6 +47,8 @@ __global__ void __launch_bounds__(kBsThreads, DEC ? kBsCtasPerSmDec : kBsCtasPer
     __shared__ __align__(16) uint32_t keys_s[(NR + 1) * bs::kKeyStepWords];
     for (int i = threadIdx.x; i < (NR + 1) * bs::kKeyStepWords; i += blockDim.x) keys_s[i] = a.planes[i];
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t h = lane & 1u, g = lane >> 1;
     const bs::HalfKeys keys{keys_s + bs::kKeyHalfWords * h};
@@ -121,8 +124,7 @@ int launch_bitsliced(const EcbArgs& e, const uint32_t* enc_rk, int nr, Mode mode
     uint64_t grid = (uint64_t)info.sms * per_sm;
     const uint64_t need = (tiles + warps_per_cta - 1) / warps_per_cta;
     if (need < grid) grid = need;
-    fn<<<(unsigned)grid, kBsThreads, 0, stream>>>(a);
-    err = cudaGetLastError();
+    err = launch_overlapped(fn, (unsigned)grid, kBsThreads, 0, stream, a);
     if (err != cudaSuccess) return fail(AES_ERR_CUDA, "bitsliced kernel launch: %s", cudaGetErrorString(err));
     return AES_OK;
 }

@@ -1,0 +1,56 @@
+// Launches that overlap the kernel before them in their stream (programmatic
+// dependent launch), for every kernel that runs once per call.
+//
+// A stream starts a kernel once the one before it has ended and flushed; between
+// two short kernels that gap is longer than the kernels (4.1 us per call for 4 KiB, of
+// which the kernel itself takes 2.2, and 6.15 us for 1 MiB).  A kernel launched here
+// may start while its predecessor still runs or drains: it fills its shared-memory
+// tables, which depend on no earlier work, and then waits (pdl_wait) for everything
+// before it in the stream to have ended and its writes to be visible.  Measured on a
+// stream of such calls, before and after: 4 KiB 4.10 -> 2.6 us (host bound), 1 MiB 6.15 ->
+// 3.07, 9 MiB 15.8 -> 12.4, 64 MiB 79.9 -> 76.6.  Filling the tables before the wait
+// instead of after it is 0.7 us of that, and costs a call on its own nothing that
+// could be measured (the first block's load no longer overlaps the fill).
+//
+// Every kernel launched here calls pdl_wait in every thread before it touches
+// global memory other than constants of the library, and pdl_trigger once.  A
+// predecessor that never triggers (another library's kernel) ends first, as without
+// the attribute; so does any kernel that follows with a plain launch.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace gbaes {
+
+#ifdef __CUDACC__
+// Waits until every earlier operation of the stream has ended and its writes are visible.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Lets the next kernel of the stream start (once every CTA has called this or ended).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// fn<<<grid, threads, smem, stream>>>(a), overlapping its predecessor.  A stream
+// being captured gets a plain launch, so that a captured graph has ordinary edges.
+template <class Args>
+cudaError_t launch_overlapped(void (*fn)(Args), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
+                              const Args& a) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+        cudaGetLastError();  // (the legacy stream beside a capture: the launch reports it)
+    } else if (cap == cudaStreamCaptureStatusNone) {
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, fn, a);
+}
+#endif
+
+}  // namespace gbaes

@@ -420,3 +420,61 @@ def test_size_dispatch_and_balanced_shapes_vs_oracle(gbaes, decrypt):
                     out = gbaes.ecb_ex(k, x, decrypt=decrypt, kernel=kid, blocks_per_thread=bpt)
                     assert np.array_equal(host(out), want), (n, kid, bpt)
     assert gbaes.device_status() == 0
+
+
+@pytest.mark.parametrize("captured", (False, True))
+@pytest.mark.parametrize("n", (1, 4096, 19_456, 19_457, 65_536, 400_000))
+def test_dependent_calls_back_to_back(gbaes, n, captured):
+    """Calls that each take the one before's output, in place and without a wait
+    between them, mixed with torch's own kernels and batches: each must see the
+    finished output of its predecessor (a kernel may start while the one before
+    it in the stream still runs).  Undoing every step gives the input back, and
+    the state in the middle is the oracle's."""
+    rng = np.random.default_rng(n)
+    raw = [rng.integers(0, 256, b // 8, dtype=np.uint8).tobytes() for b in BITS]
+    ks = [gbaes.Key(r) for r in raw]
+    data = rng.integers(0, 256, 16 * n, dtype=np.uint8)
+    iv = bytes(range(16))
+    cut = n // 2
+    descs = [gbaes.make_descs([0, 16 * cut], [0, 16 * cut], [cut, n - cut], [0, 2], [d, 1 - d]) for d in (0, 1)]
+    plans = [gbaes.BatchPlan(d, ks) for d in descs]
+    steps = 6
+    x = dev(data)
+    mid = torch.empty_like(x)
+
+    def chain():
+        for i in range(steps):
+            gbaes.encrypt_ecb(ks[i % 3], x, x)
+            gbaes.ctr_xcrypt(ks[(i + 1) % 3], iv, x, x, first_block=i)
+            plans[0].launch(x, x)
+            x.bitwise_xor_(i + 1)
+        mid.copy_(x)
+        for i in reversed(range(steps)):
+            x.bitwise_xor_(i + 1)
+            plans[1].launch(x, x)
+            gbaes.ctr_xcrypt(ks[(i + 1) % 3], iv, x, x, first_block=i)
+            gbaes.decrypt_ecb(ks[i % 3], x, x)
+
+    if captured:
+        s = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s):
+            chain()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            chain()
+        g.replay()
+        g.replay()
+    else:
+        chain()
+    assert np.array_equal(host(x), data)
+    want = data
+    for i in range(steps):
+        want = oracle.ecb(raw[i % 3], BITS[i % 3], want)
+        shifted = ((int.from_bytes(iv, "big") + i) % (1 << 128)).to_bytes(16, "big")
+        want = oracle.ctr(raw[(i + 1) % 3], BITS[(i + 1) % 3], shifted, want)
+        parts = [oracle.ecb(raw[0], 128, want[:16 * cut])] if cut else []
+        want = np.concatenate(parts + [oracle.ecb(raw[2], 256, want[16 * cut:], decrypt=True)]) ^ np.uint8(i + 1)
+    assert np.array_equal(host(mid), want)
+    assert gbaes.device_status() == 0
