@@ -26,6 +26,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <set>
@@ -306,16 +307,19 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
 
 static int group_of(int nr, int dir) { return dir * 3 + (nr == 10 ? 0 : nr == 12 ? 1 : 2); }
 
-// Validates the descriptors and lays out groups, tiles and key slots.
-int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx,
-                           uint32_t tile_blocks, bool with_keys, HostPlan* P) {
+// Validates the descriptors and lays out groups and tiles: one pass checks and
+// counts, a second writes each message to its place.
+int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx, uint32_t tile_blocks,
+                    HostPlan* P) {
     if (nmsg && !d) return fail(AES_ERR_ARG, "message descriptors are NULL");
     if (nctx && !ctxs) return fail(AES_ERR_ARG, "key contexts are NULL");
     if (nmsg > 0xFFFFFFF0u) return fail(AES_ERR_ARG, "too many messages (%zu)", nmsg);
     if (tile_blocks == 0) return fail(AES_ERR_ARG, "tile size is zero");
     for (size_t i = 0; i < nctx; ++i)
         if (!ctxs[i] || ctxs[i]->magic != kCtxMagic) return fail(AES_ERR_ARG, "ctxs[%zu] is not a valid aes_ctx", i);
-    std::vector<uint32_t> order[kGroups];
+    uint32_t count[kGroups] = {};
+    uint64_t blocks[kGroups] = {};
+    std::vector<uint8_t> group(nmsg);  // kGroups: no blocks
     for (size_t i = 0; i < nmsg; ++i) {
         const aes_msg_desc& m = d[i];
         if (m.key_index >= nctx) return fail(AES_ERR_ARG, "message %zu: key_index %u >= %zu", i, m.key_index, nctx);
@@ -325,54 +329,49 @@ int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ct
         const uint64_t bytes = m.nblocks * 16;
         if (m.in_off > UINT64_MAX - bytes || m.out_off > UINT64_MAX - bytes)
             return fail(AES_ERR_ARG, "message %zu: offset + length overflows", i);
+        group[i] = kGroups;
         if (m.nblocks == 0) continue;
         P->in_extent = std::max<uint64_t>(P->in_extent, m.in_off + bytes);
         P->out_extent = std::max<uint64_t>(P->out_extent, m.out_off + bytes);
-        order[group_of(ctxs[m.key_index]->nr, (int)m.decrypt)].push_back((uint32_t)i);
+        const int g = group_of(ctxs[m.key_index]->nr, (int)m.decrypt);
+        group[i] = (uint8_t)g;
+        ++count[g];
+        blocks[g] += m.nblocks;
     }
     P->tile_blocks = tile_blocks;
-    uint64_t tiles = 0;
+    uint64_t tiles = 0, msgs = 0;
+    uint32_t next[kGroups];  // where each group's next message goes
     for (int g = 0; g < kGroups; ++g) {
         GroupDev& G = P->groups[g];
         G.nr = g % 3 == 0 ? 10 : g % 3 == 1 ? 12 : 14;
         G.dir = g / 3;
-        G.msg_start = (uint32_t)P->msgs.size();
-        uint64_t blk = 0;
-        for (uint32_t i : order[g]) {
-            const aes_msg_desc& m = d[i];
-            MsgDev md;
-            md.blk_start = blk;
-            md.in_blk = m.in_off >> 4;
-            md.out_blk = m.out_off >> 4;
-            md.key_slot = 2u * m.key_index + m.decrypt;
-            md.src = i;
-            P->msgs.push_back(md);
-            blk += m.nblocks;
-        }
-        G.msg_end = (uint32_t)P->msgs.size();
-        G.blocks = blk;
-        const uint64_t gt = (blk + tile_blocks - 1) / tile_blocks;
+        next[g] = G.msg_start = (uint32_t)msgs;
+        G.msg_end = (uint32_t)(msgs += count[g]);
+        G.blocks = blocks[g];
+        const uint64_t gt = (blocks[g] + tile_blocks - 1) / tile_blocks;
         // headroom: warps read the counter past the last tile, offset by the fixed first tiles
         if (tiles + gt > 0xFFFF0000u) return fail(AES_ERR_ARG, "batch needs too many tiles");
         G.tile_start = (uint32_t)tiles;
-        G.tile_end = (uint32_t)(tiles + gt);
-        // first message of each tile: walk the group's messages once
-        uint32_t m = G.msg_start;
-        for (uint64_t lt = 0; lt < gt; ++lt) {
-            const uint64_t first = lt * tile_blocks;
-            while (m + 1 < G.msg_end && P->msgs[m + 1].blk_start <= first) ++m;
-            P->tile_msg.push_back(m);
-        }
-        tiles += gt;
-        P->total_blocks += blk;
+        G.tile_end = (uint32_t)(tiles += gt);
+        P->total_blocks += blocks[g];
+        blocks[g] = 0;  // from here: blocks of the messages placed
     }
     P->ntiles = (uint32_t)tiles;
-    if (with_keys) {
-        P->keys.assign(2 * nctx * kSlotWords, 0u);
-        for (size_t i = 0; i < nctx; ++i) {
-            const int words = 4 * (ctxs[i]->nr + 1);
-            memcpy(&P->keys[(2 * i) * kSlotWords], ctxs[i]->enc_rk, 4 * words);
-            memcpy(&P->keys[(2 * i + 1) * kSlotWords], ctxs[i]->dec_rk, 4 * words);
+    P->msgs.resize(msgs);
+    for (size_t i = 0; i < nmsg; ++i) {
+        const int g = group[i];
+        if (g == kGroups) continue;
+        const aes_msg_desc& m = d[i];
+        P->msgs[next[g]++] = MsgDev{blocks[g], m.in_off >> 4, m.out_off >> 4, 2u * m.key_index + m.decrypt, (uint32_t)i};
+        blocks[g] += m.nblocks;
+    }
+    P->tile_msg.resize(tiles);
+    for (const GroupDev& G : P->groups) {  // first message of each tile: walk the group's messages once
+        uint32_t m = G.msg_start;
+        uint64_t first = 0;
+        for (uint32_t t = G.tile_start; t < G.tile_end; ++t, first += tile_blocks) {
+            while (m + 1 < G.msg_end && P->msgs[m + 1].blk_start <= first) ++m;
+            P->tile_msg[t] = m;
         }
     }
     return AES_OK;
@@ -403,6 +402,51 @@ namespace gbaes {
 constexpr uint32_t kPlanMagic = 0x504c414eu;  // "PLAN"
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// The device tables of a plan, in one piece: the counter (256 bytes), two
+// schedules per context, the messages, the tiles.
+struct Tables {
+    static constexpr size_t off_keys = 256;
+    size_t off_msgs, off_tiles, bytes;
+    Tables(const HostPlan& H, size_t nctx) {
+        off_msgs = off_keys + nctx * 2 * kSlotWords * 4;
+        off_tiles = off_msgs + align256(H.msgs.size() * sizeof(MsgDev));
+        bytes = off_tiles + align256(H.tile_msg.size() * 4 + 4);
+    }
+    // Their host copy (bytes long).
+    std::unique_ptr<uint8_t[]> image(const HostPlan& H, const aes_ctx* const* ctxs, size_t nctx) const {
+        std::unique_ptr<uint8_t[]> img(new uint8_t[bytes]);
+        memset(img.get(), 0, off_keys);
+        for (size_t i = 0; i < nctx; ++i) {
+            const size_t n = 16 * (size_t)(ctxs[i]->nr + 1), slot = 4 * kSlotWords;
+            uint8_t* p = img.get() + off_keys + 2 * i * slot;
+            memcpy(p, ctxs[i]->enc_rk, n);
+            memset(p + n, 0, slot - n);
+            memcpy(p + slot, ctxs[i]->dec_rk, n);
+            memset(p + slot + n, 0, slot - n);
+        }
+        put(img.get(), off_msgs, off_tiles, H.msgs.data(), H.msgs.size() * sizeof(MsgDev));
+        put(img.get(), off_tiles, bytes, H.tile_msg.data(), H.tile_msg.size() * 4);
+        return img;
+    }
+    // Points a launch's arguments at the tables at dev.
+    void fill_args(const HostPlan& H, uint8_t* dev, int* status, BatchArgs* a) const {
+        a->msgs = (const MsgDev*)(dev + off_msgs);
+        a->keys = (const uint4*)(dev + off_keys);
+        a->tile_msg = (const uint32_t*)(dev + off_tiles);
+        a->counter = (unsigned*)dev;
+        a->status = status;
+        a->ntiles = H.ntiles;
+        a->tile_blocks = H.tile_blocks;
+        memcpy(a->groups, H.groups, sizeof a->groups);
+    }
+
+  private:
+    static void put(uint8_t* img, size_t from, size_t to, const void* src, size_t n) {
+        if (n) memcpy(img + from, src, n);
+        memset(img + from + n, 0, to - from - n);
+    }
+};
 
 using BatchKernel = void (*)(const BatchArgs);
 
@@ -564,7 +608,7 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
     // (less work left over in the last wave); at 4 blocks per thread 256-block tiles lost (0.8705 against
     // 0.8745 at 512).
     const uint32_t tile_blocks = std::min(128u * (uint32_t)blocks_per_thread, kPlanTileMax);
-    if (build_host_plan(msgs, nmsg, ctxs, nctx, tile_blocks, true, &P->host)) {
+    if (build_host_plan(msgs, nmsg, ctxs, nctx, tile_blocks, &P->host)) {
         delete P;
         return nullptr;
     }
@@ -574,21 +618,15 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
         return nullptr;
     }
     const HostPlan& H = P->host;
-    const size_t off_keys = 256;
-    const size_t off_msgs = off_keys + align256(H.keys.size() * 4);
-    const size_t off_tiles = off_msgs + align256(H.msgs.size() * sizeof(MsgDev));
-    P->dev_bytes = off_tiles + align256(H.tile_msg.size() * 4 + 4);
+    const Tables tables(H, nctx);
+    P->dev_bytes = tables.bytes;
     cudaError_t e = cudaMalloc(&P->dev_buf, P->dev_bytes);
     if (e != cudaSuccess) {
         fail(AES_ERR_NOMEM, "cudaMalloc(%zu): %s", P->dev_bytes, cudaGetErrorString(e));
         delete P;
         return nullptr;
     }
-    std::vector<uint8_t> img(P->dev_bytes, 0);
-    if (!H.keys.empty()) memcpy(img.data() + off_keys, H.keys.data(), H.keys.size() * 4);
-    if (!H.msgs.empty()) memcpy(img.data() + off_msgs, H.msgs.data(), H.msgs.size() * sizeof(MsgDev));
-    if (!H.tile_msg.empty()) memcpy(img.data() + off_tiles, H.tile_msg.data(), H.tile_msg.size() * 4);
-    e = cudaMemcpy(P->dev_buf, img.data(), P->dev_bytes, cudaMemcpyHostToDevice);
+    e = cudaMemcpy(P->dev_buf, tables.image(H, ctxs, nctx).get(), P->dev_bytes, cudaMemcpyHostToDevice);
     int* status = nullptr;
     if (e != cudaSuccess || device_status_word(&status)) {
         fail(AES_ERR_CUDA, "uploading the batch plan: %s", cudaGetErrorString(e));
@@ -598,14 +636,7 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
     }
     BatchArgs& a = P->args;
     memset(&a, 0, sizeof a);
-    a.msgs = (const MsgDev*)(P->dev_buf + off_msgs);
-    a.keys = (const uint4*)(P->dev_buf + off_keys);
-    a.tile_msg = (const uint32_t*)(P->dev_buf + off_tiles);
-    a.counter = (unsigned*)P->dev_buf;
-    a.status = status;
-    a.ntiles = H.ntiles;
-    a.tile_blocks = H.tile_blocks;
-    memcpy(a.groups, H.groups, sizeof a.groups);
+    tables.fill_args(H, P->dev_buf, status, &a);
     if (H.ntiles) {
         const BatchSchedule sch = current_schedule(H, P->threads, P->bpt);
         a.split = sch.split;
@@ -716,25 +747,19 @@ int aes_ecb_batch(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* c
                     "use aes_batch_plan_launch_graph");
     HostPlan H;
     const OneShot shape = one_shot_shape(msgs, nmsg);
-    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, true, &H);
+    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, &H);
     if (rc) return rc;
     if (H.ntiles == 0) return AES_OK;
     rc = check_bases(H, in_base, in_bytes, out_base, out_bytes);
     if (rc) return rc;
     // Stream-ordered scratch: plan tables live only as long as the launch.
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t off_keys = 256;
-    const size_t off_msgs = off_keys + align256(H.keys.size() * 4);
-    const size_t off_tiles = off_msgs + align256(H.msgs.size() * sizeof(MsgDev));
-    const size_t bytes = off_tiles + align256(H.tile_msg.size() * 4 + 4);
-    std::vector<uint8_t> img(bytes, 0);
-    memcpy(img.data() + off_keys, H.keys.data(), H.keys.size() * 4);
-    memcpy(img.data() + off_msgs, H.msgs.data(), H.msgs.size() * sizeof(MsgDev));
-    memcpy(img.data() + off_tiles, H.tile_msg.data(), H.tile_msg.size() * 4);
+    const Tables tables(H, nctx);
     uint8_t* buf = nullptr;
-    e = cudaMallocAsync((void**)&buf, bytes, s);
-    if (e != cudaSuccess) return fail(AES_ERR_NOMEM, "cudaMallocAsync(%zu): %s", bytes, cudaGetErrorString(e));
-    e = cudaMemcpyAsync(buf, img.data(), bytes, cudaMemcpyHostToDevice, s);  // pageable: staged before return
+    e = cudaMallocAsync((void**)&buf, tables.bytes, s);
+    if (e != cudaSuccess) return fail(AES_ERR_NOMEM, "cudaMallocAsync(%zu): %s", tables.bytes, cudaGetErrorString(e));
+    const auto img = tables.image(H, ctxs, nctx);
+    e = cudaMemcpyAsync(buf, img.get(), tables.bytes, cudaMemcpyHostToDevice, s);  // pageable: staged before return
     int* status = nullptr;
     if (e != cudaSuccess || device_status_word(&status)) {
         cudaFreeAsync(buf, s);
@@ -744,14 +769,7 @@ int aes_ecb_batch(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* c
     memset(&a, 0, sizeof a);
     a.in = (const uint4*)in_base;
     a.out = (uint4*)out_base;
-    a.msgs = (const MsgDev*)(buf + off_msgs);
-    a.keys = (const uint4*)(buf + off_keys);
-    a.tile_msg = (const uint32_t*)(buf + off_tiles);
-    a.counter = (unsigned*)buf;
-    a.status = status;
-    a.ntiles = H.ntiles;
-    a.tile_blocks = H.tile_blocks;
-    memcpy(a.groups, H.groups, sizeof a.groups);
+    tables.fill_args(H, buf, status, &a);
     rc = launch_batch_kernel(H, a, shape.threads, shape.bpt, s);
     cudaFreeAsync(buf, s);
     return rc;
@@ -761,7 +779,7 @@ int aes_batch_tiles(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const*
                     uint32_t* first_msg, size_t cap) {
     if (tile_blocks <= 0) return fail(AES_ERR_ARG, "tile_blocks must be positive");
     HostPlan H;
-    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, (uint32_t)tile_blocks, false, &H);
+    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, (uint32_t)tile_blocks, &H);
     if (rc) return rc;
     if (first_msg) {
         if (cap < H.ntiles) return fail(AES_ERR_ARG, "first_msg holds %zu entries, the batch has %u tiles", cap, H.ntiles);
@@ -823,53 +841,40 @@ int aes_ecb_batch_noalloc(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* 
                           const void* in_base, size_t in_bytes, void* out_base, size_t out_bytes, void* stream) {
     HostPlan H;
     OneShot shape = one_shot_shape(msgs, nmsg);
-    size_t off_keys = 256, off_msgs = 0, off_tiles = 0, bytes = 0;  // [0, 256): tile counter, uploaded as zero
-    int rc = AES_OK;
-    for (;;) {
-        rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, true, &H);
-        if (rc) return rc;
-        off_msgs = off_keys + align256(H.keys.size() * 4);
-        off_tiles = off_msgs + align256(H.msgs.size() * sizeof(MsgDev));
-        bytes = off_tiles + align256(H.tile_msg.size() * 4 + 4);
-        if (bytes <= kNoAllocScratchBytes || shape.tile_blocks == kOneShotTileMax) break;
+    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, &H);
+    if (rc) return rc;
+    if (Tables(H, nctx).bytes > kNoAllocScratchBytes && shape.tile_blocks != kOneShotTileMax) {
         shape.tile_blocks = kOneShotTileMax;  // the smallest tables
         H = HostPlan();
+        rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, &H);
+        if (rc) return rc;
     }
     if (H.ntiles == 0) return AES_OK;
     rc = check_bases(H, in_base, in_bytes, out_base, out_bytes);
     if (rc) return rc;
-    if (bytes > kNoAllocScratchBytes)
+    const Tables tables(H, nctx);
+    if (tables.bytes > kNoAllocScratchBytes)
         return fail(AES_ERR_ARG,
                     "batch needs %zu bytes of tables (keys: 512 B per context; 32 B per message; 4 B per tile), "
                     "the allocation-free entry point holds at most %zu",
-                    bytes, kNoAllocScratchBytes);
+                    tables.bytes, kNoAllocScratchBytes);
     uint8_t* buf = nullptr;
     rc = noalloc_scratch(&buf);
     if (rc) return rc;
     int* status = nullptr;
     rc = device_status_word(&status);
     if (rc) return rc;
-    std::vector<uint8_t> img(bytes, 0);  // host staging only; the counter word stays zero
-    memcpy(img.data() + off_keys, H.keys.data(), H.keys.size() * 4);
-    memcpy(img.data() + off_msgs, H.msgs.data(), H.msgs.size() * sizeof(MsgDev));
-    memcpy(img.data() + off_tiles, H.tile_msg.data(), H.tile_msg.size() * 4);
+    const auto img = tables.image(H, ctxs, nctx);  // host staging only; the counter words are zero
     cudaStream_t s = (cudaStream_t)stream;
     // Stream-ordered after earlier work on `stream`; from pageable memory the
     // call returns once the image is staged, so img may be released after it.
-    cudaError_t e = cudaMemcpyAsync(buf, img.data(), bytes, cudaMemcpyHostToDevice, s);
+    cudaError_t e = cudaMemcpyAsync(buf, img.get(), tables.bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "uploading the batch tables: %s", cudaGetErrorString(e));
     BatchArgs a;
     memset(&a, 0, sizeof a);
     a.in = (const uint4*)in_base;
     a.out = (uint4*)out_base;
-    a.msgs = (const MsgDev*)(buf + off_msgs);
-    a.keys = (const uint4*)(buf + off_keys);
-    a.tile_msg = (const uint32_t*)(buf + off_tiles);
-    a.counter = (unsigned*)buf;
-    a.status = status;
-    a.ntiles = H.ntiles;
-    a.tile_blocks = H.tile_blocks;
-    memcpy(a.groups, H.groups, sizeof a.groups);
+    tables.fill_args(H, buf, status, &a);
     return launch_batch_kernel(H, a, shape.threads, shape.bpt, s);
 }
 

@@ -50,7 +50,6 @@ struct BatchArgs {
 struct HostPlan {
     std::vector<MsgDev> msgs;
     std::vector<uint32_t> tile_msg;
-    std::vector<uint32_t> keys;  // 2 * nctx slots of kSlotWords words
     GroupDev groups[kGroups];
     uint32_t ntiles = 0;
     uint32_t tile_blocks = 0;
@@ -59,9 +58,9 @@ struct HostPlan {
     uint64_t out_extent = 0;  // bytes from out_base the plan writes
 };
 
-// Validates descriptors and lays out groups, tiles and (optionally) key slots.
+// Validates descriptors and lays out groups and tiles.
 int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx, uint32_t tile_blocks,
-                    bool with_keys, HostPlan* P);
+                    HostPlan* P);
 
 // How one batched launch shares its tiles among the GPU's warps (BatchArgs::split, enc_ctas).
 struct BatchSchedule {

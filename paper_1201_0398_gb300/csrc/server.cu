@@ -722,7 +722,7 @@ static int launch_slot(aes_server* S, Slot& slot) {
     // batch) p50 / p99 went from 32.9 / 54.3 to 26.3 / 41.6 us, at 800k from 56.0 / 101.5
     // to 35.5 / 54.9.
     const uint32_t tb = kServerTileBlocks;
-    int rc = build_host_plan(d.data(), d.size(), S->key_ptrs.data(), S->key_ptrs.size(), tb, false, &H);
+    int rc = build_host_plan(d.data(), d.size(), S->key_ptrs.data(), S->key_ptrs.size(), tb, &H);
     if (rc) return rc;
     if (H.ntiles == 0) return AES_OK;
     const size_t off_msgs = 256;
@@ -1361,7 +1361,9 @@ static int enqueue(aes_server* S, const aes_server_request& r, double arrival) {
 static void producer_main(aes_server* S) {
     pthread_setname_np(pthread_self(), "gbaes-replay");
     if (!S->dryrun) cudaSetDevice(S->device);  // (the stack registration and pool chunks use its context)
-    const PinnedStackTop stack_top(!S->dryrun);
+    // Page-locking the stack takes ~80 us: worth it for a replay that lasts.
+    const bool lasts = !S->replay_reqs.empty() && S->replay_reqs.back().arrival_s > 0.05;
+    const PinnedStackTop stack_top(!S->dryrun && lasts);
     if (S->cfg.flags & AES_SERVER_PIN_THREADS) S->producer_cpu = pin_thread(1);
     const double start = S->now();
     S->replay_start = start;
@@ -1718,10 +1720,15 @@ int aes_server_replay_join(aes_server* S, int stop_early) {
 
 int aes_server_drain(aes_server* S, double timeout_s) {
     if (!S || S->magic != kServerMagic) return fail(AES_ERR_ARG, "invalid aes_server");
-    const double until = S->now() + timeout_s;
+    const double begin = S->now(), until = begin + timeout_s;
     while (S->finished.load() < S->submitted.load() || S->producer_running.load()) {
-        if (timeout_s >= 0 && S->now() > until) return fail(AES_ERR_STATE, "drain timed out");
-        std::this_thread::sleep_for(std::chrono::microseconds(50));
+        const double t = S->now();
+        if (timeout_s >= 0 && t > until) return fail(AES_ERR_STATE, "drain timed out");
+        // A sleep of 50 us lasts about 100: a short drain only yields.
+        if (t - begin < 200e-6)
+            std::this_thread::yield();
+        else
+            std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
     return AES_OK;
 }
