@@ -61,8 +61,8 @@ extern "C" {
                                          memory, cheap to fill; lookups may meet bank conflicts), any
                                          size; its launch shape is its own (threads and
                                          blocks_per_thread are ignored) */
-#define AES_KERNEL_TABLE_REPLICATED 3 /* T-table kernel with 32 lane copies of each table (bank-conflict
-                                         free, 128-160 KiB to fill per CTA), any size */
+#define AES_KERNEL_TABLE_REPLICATED 3 /* T-table kernel with 32 lane copies of its table (bank-conflict
+                                         free, 32 KiB to fill per CTA), any size */
 
 /* Counter layouts for aes_ctr_xcrypt (Section 3, CTR mode). */
 #define AES_CTR_BE128 0     /* IV is one big-endian 128-bit integer (NIST SP 800-38A) */

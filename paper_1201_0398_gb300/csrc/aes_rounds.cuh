@@ -1,17 +1,29 @@
-// Device-side AES rounds in the T-table form of Eq. 1, shared by the block
-// kernels (ecb_table.cu) and the batched kernel (batch.cu).
+// Device-side AES rounds in the T-table form of Eq. 1, shared by every table
+// kernel.
 //
-// Shared-memory layout (bank-conflict free, one PRMT per lookup address):
-//   * Every table is replicated 32 times; lane l reads copy l, so lane l always
-//     hits bank l whatever byte it looks up.
-//   * Region r (64 KiB) holds T_{2r} and T_{2r+1}: word 64*x + 32*slot + l is
-//     T_{2r+slot}[x] for lane l, i.e. byte address x<<8 | slot<<7 | l<<2.  A
-//     __byte_perm drops state byte k into address byte 1 beside a per-lane
-//     constant (l<<2 | slot<<7 | the region base, which is 64 KiB aligned).
-//     Region 1 is reached through the load's immediate offset.
-//   * The inverse cipher adds the inverse S-box for its last round (32x
-//     replicated, 32 words per entry) after the two regions.
-// T_k[x] = rotl(T_0[x], 8k) (Eq. 1's four tables are rotations of one).
+// Shared-memory layout: one table per direction, 32 KiB.  Entry x of T_0 is stored
+// 32 times side by side (128 bytes at 128 x); lane l reads copy l, so lane l always
+// hits the same bank whatever byte it looks up.  The other three tables of Eq. 1
+// are rotations, T_k[x] = rotl(T_0[x], 8k), and cost one byte permute of the
+// entry read.
+//
+// A lookup address is one dp4a: byte k of a state word times 128 plus the lane's
+// base, the other three bytes times 0.  dp4a runs on the multiply-add pipe at the
+// ALU's rate (64 lanes/clk/SM), beside it: dp4a and lop3 in turn issue 3.63 warp
+// instructions per clock and SM, prmt and lop3 1.99.  A round of a warp is 16
+// lookups (16 clocks of the shared-memory pipe, the bound), 16 dp4a (8 clocks), and
+// 12 permutes and 8 three-input XORs (10 clocks of the ALU).
+//
+// Measured, AES-128, 1 GiB, cycles of an SM per 32 blocks (160 are lookups):
+//   four tables of 32 KiB, PRMT addresses (64 KiB aligned)   177  (909 GB/s)
+//   the same with dp4a addresses                             177
+//   four tables at the start of the shared-memory window     172
+//   one table, two CTAs of 512 threads per SM                172  (937 GB/s)
+//   one table 128 KiB into the window                        179
+// The global loads and stores (about 12 of the 172) share the L1 data stage with the
+// lookups, and tables far into the window get more in their way.  One table is also
+// a quarter of the fill (256 store cycles instead of 1,024), lets two CTAs share an
+// SM, and leaves room for both directions' tables at once.
 #pragma once
 
 #include <cstdint>
@@ -24,10 +36,7 @@ namespace gbaes {
 // Source of the shared-memory fills, read through the read-only global path.
 static __device__ AesTables g_tab = make_aes_tables();
 
-constexpr uint32_t kRegion = 0x10000u;                 // one 64 KiB region: two tables
-constexpr uint32_t kEncBytes = 2 * kRegion;            // T0|T1, T2|T3
-constexpr uint32_t kSiOffset = 2 * kRegion;            // inverse cipher: inverse S-box
-constexpr uint32_t kDecBytes = 2 * kRegion + 0x8000u;  // + 256 entries x 32 lanes x 4 B
+constexpr uint32_t kTableBytes = 0x8000u;  // 256 entries x 32 lanes x 4 B
 
 __device__ __forceinline__ uint32_t lds(uint32_t addr) {
     uint32_t v;
@@ -47,11 +56,10 @@ __device__ __forceinline__ void sts(uint32_t addr, uint32_t v) {
 }
 
 // Streaming 16-byte global load that does not allocate in L1: the input is read
-// once, and keeping it out of L1 keeps its fills out of the SRAM the
-// shared-memory tables live in.
+// once.  Volatile, so that a load meant to go out before the rounds stays there.
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     uint4 v;
-    asm("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
         : "l"(p));
     return v;
@@ -59,30 +67,19 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
 
 __device__ __forceinline__ uint32_t smem_base(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ uint32_t dynamic_smem_bytes() {
-    uint32_t dyn;
-    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-    return dyn;
-}
-
-// 64 KiB-aligned start of the table layout inside the dynamic window.
-__device__ __forceinline__ uint32_t table_base(uint32_t base) { return (base + (kRegion - 1)) & ~(kRegion - 1); }
-
-// Fill store: ordered before the tables' first use by the __syncthreads that
-// follows every fill, so it needs no compiler memory clobber (which would keep
-// the next entry's global load from being issued early).
+// Fill store: ordered before the table's first use by the barrier that follows
+// every fill, so it needs no compiler memory clobber (which would keep the next
+// entry's global load from being issued early).
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t v) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(v));
 }
 
-// Writes the tables of one direction into shared memory at A; threads tid =
-// 0..nt-1 take part (fill_tables: the whole CTA), and the caller synchronises
-// them afterwards.  Pair p = (entry x = p/4, table k = p%4): its 32 lane copies
-// are 128 contiguous bytes at region k/2, slot k%2, written as eight 16-byte
-// stores in an order rotated by p, so the 8 threads of each quarter-warp hit 8
-// different bank groups.  A thread loads the entries of up to four pairs before
-// storing any, so small CTAs (many pairs per thread) overlap the global loads.
-__device__ __forceinline__ void fill_tables_n(uint32_t A, bool decrypt, uint32_t tid, uint32_t nt) {
+// Writes one direction's table at A (16-byte aligned); threads tid = 0..nt-1 take
+// part and the caller synchronises them.  Four threads share an entry's 128 bytes:
+// thread p writes two 16-byte pieces of entry p / 4, the pieces rotated so that the
+// 8 threads of a quarter-warp's store hit 8 different bank groups.  A thread loads
+// up to four entries before storing any.
+__device__ __forceinline__ void fill_table(uint32_t A, bool decrypt, uint32_t tid, uint32_t nt) {
     const uint32_t* t0 = decrypt ? g_tab.td0 : g_tab.te0;
     for (uint32_t p0 = tid; p0 < 1024u; p0 += 4u * nt) {
         uint32_t v[4];
@@ -95,121 +92,64 @@ __device__ __forceinline__ void fill_tables_n(uint32_t A, bool decrypt, uint32_t
         for (uint32_t u = 0; u < 4; ++u) {
             const uint32_t p = p0 + u * nt;
             if (p < 1024u) {
-                const uint32_t k = p & 3u;
-                const uint32_t val = __funnelshift_l(v[u], v[u], 8u * k);  // T_k[x] = rotl(T_0[x], 8k)
-                const uint32_t base = A + (k >> 1) * kRegion + (p >> 2) * 256u + (k & 1u) * 128u;
-#pragma unroll
-                for (uint32_t j = 0; j < 8; ++j) sts128(base + 16u * ((j + p) & 7u), val);
-            }
-        }
-    }
-    if (decrypt) {
-        for (uint32_t x0 = tid; x0 < 256u; x0 += 4u * nt) {
-            uint32_t v[4];
-#pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) {
-                const uint32_t x = x0 + u * nt;
-                v[u] = x < 256u ? __ldg(g_tab.si4 + x) : 0u;
-            }
-#pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) {
-                const uint32_t x = x0 + u * nt;
-                if (x < 256u) {
-                    const uint32_t base = A + kSiOffset + x * 128u;
-#pragma unroll
-                    for (uint32_t j = 0; j < 8; ++j) sts128(base + 16u * ((j + x) & 7u), v[u]);
-                }
+                const uint32_t piece = 2u * (p & 3u) + ((p >> 2) & 1u);
+                const uint32_t base = A + (p >> 2) * 128u;
+                sts128(base + 16u * piece, v[u]);
+                sts128(base + 16u * (piece ^ 1u), v[u]);
             }
         }
     }
 }
 
-__device__ __forceinline__ void fill_tables(uint32_t A, bool decrypt) { fill_tables_n(A, decrypt, threadIdx.x, blockDim.x); }
-
-// Address of T_{2*region+slot}[byte K of w] for this lane (region offset aside):
-// byte 0 <- lane constant (l<<2 | slot<<7), byte 1 <- byte K of w, bytes 2,3 <-
-// the 64 KiB-aligned base carried in the lane constant.
+// Entry [byte K of w] of T_0 for the lane whose base is L = A + 4 * lane.
 template <int K>
-__device__ __forceinline__ uint32_t taddr(uint32_t w, uint32_t lane_const) {
-    return __byte_perm(w, lane_const, 0x7604u | (K << 4));
+__device__ __forceinline__ uint32_t look(uint32_t w, uint32_t L) {
+    return lds(__dp4a(w, 0x80u << (8 * K), L));
+}
+
+// Rotation of an entry left by K bytes: T_0's entry as T_K's.
+template <int K>
+__device__ __forceinline__ uint32_t as_table(uint32_t v) {
+    return K == 0 ? v : __byte_perm(v, v, K == 1 ? 0x2103u : K == 2 ? 0x1032u : 0x0321u);
 }
 
 // (a & m) | (b & ~m): bytes of a where m is set, of b elsewhere.
 __device__ __forceinline__ uint32_t merge(uint32_t a, uint32_t b, uint32_t m) { return (a & m) | (b & ~m); }
 
-// One inner encryption round (Eq. 1).
-__device__ __forceinline__ void enc_round(uint32_t (&s)[4], uint32_t L0, uint32_t L1, uint4 k) {
+// One inner round (Eq. 1): the word that gives byte k of output word j is I_{j+k,k},
+// for the inverse cipher I_{j-k,k}.
+template <bool DECRYPT>
+__device__ __forceinline__ void round_inner(uint32_t (&s)[4], uint32_t L, uint4 k) {
+    constexpr int D = DECRYPT ? 3 : 1;
     uint32_t t[4];
     const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        uint32_t a0 = lds(taddr<0>(s[j], L0));                         // T0[I_{j,0}]
-        uint32_t a1 = lds(taddr<1>(s[(j + 1) & 3], L1));               // T1[I_{j+1,1}]
-        uint32_t a2 = lds_off<kRegion>(taddr<2>(s[(j + 2) & 3], L0));  // T2[I_{j+2,2}]
-        uint32_t a3 = lds_off<kRegion>(taddr<3>(s[(j + 3) & 3], L1));  // T3[I_{j+3,3}]
-        t[j] = a0 ^ a1 ^ a2 ^ a3 ^ kk[j];
-    }
+    for (int j = 0; j < 4; ++j)
+        t[j] = as_table<0>(look<0>(s[j], L)) ^ as_table<1>(look<1>(s[(j + D) & 3], L)) ^
+               as_table<2>(look<2>(s[(j + 2) & 3], L)) ^ as_table<3>(look<3>(s[(j + 3 * D) & 3], L)) ^ kk[j];
 #pragma unroll
     for (int j = 0; j < 4; ++j) s[j] = t[j];
 }
 
-// Last encryption round: SubBytes + ShiftRows + AddRoundKey.  S[x] is a byte of
-// each rotated table: byte 0 of T2, byte 1 of T3, byte 2 of T0, byte 3 of T1.
-__device__ __forceinline__ void enc_last(uint32_t (&s)[4], uint32_t L0, uint32_t L1, uint4 k) {
+// Last round: SubBytes + ShiftRows + AddRoundKey.  S[x] is bytes 1 and 2 of Te0's
+// entry (02 S, S, S, 03 S).  Of Td0's entry (0e Si, 09 Si, 0d Si, 0b Si) the four
+// bytes XOR to Si, as 0e ^ 09 ^ 0d ^ 0b = 01: the inverse S-box needs no table.
+template <bool DECRYPT>
+__device__ __forceinline__ void round_last(uint32_t (&s)[4], uint32_t L, uint4 k) {
+    constexpr int D = DECRYPT ? 3 : 1;
     uint32_t t[4];
     const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        uint32_t e0 = lds_off<kRegion>(taddr<0>(s[j], L0));            // T2: byte 0 = S
-        uint32_t e1 = lds_off<kRegion>(taddr<1>(s[(j + 1) & 3], L1));  // T3: byte 1 = S
-        uint32_t e2 = lds(taddr<2>(s[(j + 2) & 3], L0));               // T0: byte 2 = S
-        uint32_t e3 = lds(taddr<3>(s[(j + 3) & 3], L1));               // T1: byte 3 = S
-        uint32_t o = merge(e0, e1, 0x000000ffu);
-        o = merge(o, e2, 0x0000ffffu);
-        o = merge(o, e3, 0x00ffffffu);
-        t[j] = o ^ kk[j];
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) s[j] = t[j];
-}
-
-// One inner round of the equivalent inverse cipher: Td tables, I_{j-k,k}.
-__device__ __forceinline__ void dec_round(uint32_t (&s)[4], uint32_t L0, uint32_t L1, uint4 k) {
-    uint32_t t[4];
-    const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        uint32_t a0 = lds(taddr<0>(s[j], L0));                         // Td0[I_{j,0}]
-        uint32_t a1 = lds(taddr<1>(s[(j + 3) & 3], L1));               // Td1[I_{j-1,1}]
-        uint32_t a2 = lds_off<kRegion>(taddr<2>(s[(j + 2) & 3], L0));  // Td2[I_{j-2,2}]
-        uint32_t a3 = lds_off<kRegion>(taddr<3>(s[(j + 1) & 3], L1));  // Td3[I_{j-3,3}]
-        t[j] = a0 ^ a1 ^ a2 ^ a3 ^ kk[j];
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) s[j] = t[j];
-}
-
-// Inverse S-box entry for byte K of w: 32x replicated table, 32 words per entry.
-template <int K>
-__device__ __forceinline__ uint32_t si_lookup(uint32_t w, uint32_t L0) {
-    uint32_t b = (w >> (8 * K)) & 0xffu;
-    return lds_off<kSiOffset>((b << 7) | L0);
-}
-
-// Last round of the inverse cipher: InvShiftRows + InvSubBytes + AddRoundKey.
-__device__ __forceinline__ void dec_last(uint32_t (&s)[4], uint32_t L0, uint4 k) {
-    uint32_t t[4];
-    const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        uint32_t d0 = si_lookup<0>(s[j], L0);
-        uint32_t d1 = si_lookup<1>(s[(j + 3) & 3], L0);
-        uint32_t d2 = si_lookup<2>(s[(j + 2) & 3], L0);
-        uint32_t d3 = si_lookup<3>(s[(j + 1) & 3], L0);
-        uint32_t o = merge(d0, d1, 0x000000ffu);
-        o = merge(o, d2, 0x0000ffffu);
-        o = merge(o, d3, 0x00ffffffu);
-        t[j] = o ^ kk[j];
+        const uint32_t e0 = look<0>(s[j], L), e1 = look<1>(s[(j + D) & 3], L);
+        const uint32_t e2 = look<2>(s[(j + 2) & 3], L), e3 = look<3>(s[(j + 3 * D) & 3], L);
+        if (DECRYPT) {  // byte k: the XOR of e_k's bytes
+            const uint32_t x = __byte_perm(e0, e1, 0x5410u) ^ __byte_perm(e0, e1, 0x7632u);
+            const uint32_t y = __byte_perm(e2, e3, 0x5410u) ^ __byte_perm(e2, e3, 0x7632u);
+            t[j] = __byte_perm(x, y, 0x6420u) ^ __byte_perm(x, y, 0x7531u) ^ kk[j];
+        } else {  // byte 1 of e0, e1 and byte 2 of e2, e3 (e1's and e2's are in place)
+            t[j] = merge(merge(e1, e2, 0x0000ffffu), __byte_perm(e0, e3, 0x6001u), 0x00ffff00u) ^ kk[j];
+        }
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) s[j] = t[j];
@@ -223,39 +163,32 @@ struct ParamKeys {
     }
 };
 
-// Full cipher on BPT independent states sharing one schedule, rounds
-// interleaved across the states.
-template <int NR, bool DECRYPT, int BPT, class KS>
-__device__ __forceinline__ void cipher(uint32_t (&s)[BPT][4], const KS& ks, uint32_t L0, uint32_t L1) {
-    {
-        const uint4 k = ks.get(0);
+template <int BPT, class KS>
+__device__ __forceinline__ void whiten(uint32_t (&s)[BPT][4], const KS& ks) {
+    const uint4 k = ks.get(0);
 #pragma unroll
-        for (int b = 0; b < BPT; ++b) {
-            s[b][0] ^= k.x;
-            s[b][1] ^= k.y;
-            s[b][2] ^= k.z;
-            s[b][3] ^= k.w;
-        }
+    for (int b = 0; b < BPT; ++b) {
+        s[b][0] ^= k.x;
+        s[b][1] ^= k.y;
+        s[b][2] ^= k.z;
+        s[b][3] ^= k.w;
     }
-#pragma unroll
-    for (int r = 1; r < NR; ++r) {
+}
+
+// Rounds FIRST..NR (after the whitening) on BPT independent states sharing one
+// schedule, UNROLL rounds per iteration: unrolled in full (UNROLL >= NR) the round
+// keys are constant operands of the XORs, rolled they are loads.
+template <int NR, bool DECRYPT, int FIRST, int BPT, int UNROLL, class KS>
+__device__ __forceinline__ void rounds_from(uint32_t (&s)[BPT][4], const KS& ks, uint32_t L) {
+#pragma unroll UNROLL
+    for (int r = FIRST; r < NR; ++r) {
         const uint4 k = ks.get(r);
 #pragma unroll
-        for (int b = 0; b < BPT; ++b) {
-            if (DECRYPT)
-                dec_round(s[b], L0, L1, k);
-            else
-                enc_round(s[b], L0, L1, k);
-        }
+        for (int b = 0; b < BPT; ++b) round_inner<DECRYPT>(s[b], L, k);
     }
     const uint4 k = ks.get(NR);
 #pragma unroll
-    for (int b = 0; b < BPT; ++b) {
-        if (DECRYPT)
-            dec_last(s[b], L0, k);
-        else
-            enc_last(s[b], L0, L1, k);
-    }
+    for (int b = 0; b < BPT; ++b) round_last<DECRYPT>(s[b], L, k);
 }
 
 }  // namespace gbaes

@@ -24,7 +24,7 @@ struct AesTables {
     uint8_t inv_sbox[256];
     uint32_t te0[256];
     uint32_t td0[256];
-    uint32_t si4[256];  // inverse S-box value replicated into all four bytes
+    uint32_t si4[256];  // inverse S-box value in all four bytes (the compact tables' last round)
 };
 
 constexpr uint8_t rotl8(uint8_t v, int n) { return (uint8_t)((v << n) | (v >> (8 - n))); }

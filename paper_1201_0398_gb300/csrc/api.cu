@@ -249,7 +249,7 @@ struct Tuning {
     int bpt;
 };
 static std::atomic<int> g_kernel{AES_KERNEL_TABLE};
-static Tuning g_tuning[3][2] = {{{1024, 2}, {1024, 2}}, {{1024, 2}, {1024, 2}}, {{1024, 2}, {1024, 2}}};
+static Tuning g_tuning[3][2];  // zeros: the launcher chooses by size
 static std::mutex g_tuning_mu;
 
 static int bits_index(int bits) { return bits == 128 ? 0 : bits == 192 ? 1 : bits == 256 ? 2 : -1; }
@@ -396,8 +396,9 @@ int aes_ecb_ex(const aes_ctx* ctx, int decrypt, const void* in, void* out, size_
     Tuning t = get_tuning(ctx->bits, decrypt);
     if (threads == 0) threads = kernel == AES_KERNEL_BITSLICED ? 256 : t.threads;
     if (blocks_per_thread == 0) blocks_per_thread = t.bpt;
-    if (!valid_threads(threads)) return fail(AES_ERR_ARG, "threads %d: need a multiple of 32 in [64, 1024]", threads);
-    if (kernel != AES_KERNEL_BITSLICED && !valid_bpt(blocks_per_thread))
+    if (threads && !valid_threads(threads))
+        return fail(AES_ERR_ARG, "threads %d: need a multiple of 32 in [64, 1024]", threads);
+    if (kernel != AES_KERNEL_BITSLICED && blocks_per_thread && !valid_bpt(blocks_per_thread))
         return fail(AES_ERR_ARG, "blocks_per_thread %d: need 1, 2 or 4", blocks_per_thread);
     return run_block_op(ctx, decrypt ? kDec : kEnc, in, out, nblocks, kernel, threads, blocks_per_thread, stream,
                         nullptr, 0, 0);

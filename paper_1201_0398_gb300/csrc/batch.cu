@@ -11,13 +11,11 @@
 //    the plan records the first message it touches.  Each (key, direction)
 //    gets a slot holding its 4*(Nr+1)-word schedule.  Everything sits in one
 //    device buffer, uploaded once per plan.
-//  * Kernel.  One CTA per SM holds the shared-memory tables of aes_rounds.cuh.
+//  * Kernel.  One CTA per SM holds both directions' tables (aes_rounds.cuh).
 //    Each *warp* starts on a fixed unit (a tile, or a part of one where there are
-//    fewer tiles than warps to share them), then takes units from its
-//    direction's atomic counter on its own, so the dependent loads at the
-//    start of one warp's unit overlap the other warps' lookups; the CTA meets
-//    at a barrier only to swap its tables from one direction's set to the
-//    other's, once at most.  A warp whose unit lies in one message stages that
+//    fewer tiles than warps to share them), then takes units from an atomic
+//    counter on its own, so the dependent loads at the start of one warp's unit
+//    overlap the other warps' lookups.  A warp whose unit lies in one message stages that
 //    message's schedule in its shared-memory key slot; in other units every block
 //    finds its message from the starts of the next 32, and keys come from
 //    global memory through L1.  The round count is a run-time loop bound,
@@ -69,7 +67,7 @@ __device__ __forceinline__ uint32_t load_starts(const BatchArgs& a, const GroupD
 // end compute on zeros and store nothing, so the warp stays converged.
 template <bool DEC, int BPT>
 __device__ __forceinline__ void single_message_unit(const BatchArgs& a, const GroupDev& G, uint32_t m, uint64_t tb0,
-                                                    uint32_t n, uint32_t lane, uint32_t L0, uint32_t L1,
+                                                    uint32_t n, uint32_t lane, uint32_t L,
                                                     uint32_t kslot) {
     const uint4* mp = (const uint4*)(a.msgs + m);
     const uint4 q0 = __ldg(mp);
@@ -97,7 +95,7 @@ __device__ __forceinline__ void single_message_unit(const BatchArgs& a, const Gr
             }
             __syncwarp();
         }
-        cipher_rt<DEC, BPT>(s, SmemKeys{kslot}, G.nr, L0, L1);
+        cipher_rt<DEC, BPT>(s, SmemKeys{kslot}, G.nr, L);
 #pragma unroll
         for (int b = 0; b < BPT; ++b) {
             const uint32_t i = it + 32u * b + lane;
@@ -120,7 +118,7 @@ __device__ __forceinline__ void single_message_unit(const BatchArgs& a, const Gr
 // cipher over all of them (no divergent per-block ciphers at a boundary).
 template <bool DEC, int BPT>
 __device__ __forceinline__ void mixed_unit(const BatchArgs& a, const GroupDev& G, uint32_t m, uint32_t starts,
-                                           uint64_t tb0, uint32_t n, uint32_t lane, uint32_t L0, uint32_t L1) {
+                                           uint64_t tb0, uint32_t n, uint32_t lane, uint32_t L) {
     uint32_t wlast = __shfl_sync(0xffffffffu, starts, 31);  // the window's last entry
     for (uint32_t it = 0; it < n; it += 32u * BPT) {
         uint32_t s[BPT][4];
@@ -161,7 +159,7 @@ __device__ __forceinline__ void mixed_unit(const BatchArgs& a, const GroupDev& G
 #pragma unroll
             for (int b = 1; b < BPT; ++b)
                 if (!ok[b]) slot[b] = slot[0];  // (past the end: computes on zeros with a valid key, stores nothing)
-            cipher_rt<DEC, BPT>(s, StateKeys<BPT, kSlotWords / 4>{a.keys, slot}, G.nr, L0, L1);
+            cipher_rt<DEC, BPT>(s, StateKeys<BPT, kSlotWords / 4>{a.keys, slot}, G.nr, L);
 #pragma unroll
             for (int b = 0; b < BPT; ++b)
                 if (ok[b]) __stcs(a.out + oidx[b], make_uint4(s[b][0], s[b][1], s[b][2], s[b][3]));
@@ -174,7 +172,7 @@ __device__ __forceinline__ void mixed_unit(const BatchArgs& a, const GroupDev& G
 // consecutive blocks of the group's block space, fewer in the group's last one).
 template <bool DEC, int BPT>
 __device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupDev& G, uint32_t u, uint32_t lane,
-                                                uint32_t L0, uint32_t L1, uint32_t kslot) {
+                                                uint32_t L, uint32_t kslot) {
     const uint32_t t = u >> a.split;
     const uint32_t part = a.tile_blocks >> a.split;
     const uint64_t tb0 = (uint64_t)(t - G.tile_start) * a.tile_blocks + (u & ((1u << a.split) - 1u)) * part;
@@ -193,9 +191,9 @@ __device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupD
         }
     }
     if (!__any_sync(0xffffffffu, starts != 0u && starts < n))
-        single_message_unit<DEC, BPT>(a, G, m, tb0, n, lane, L0, L1, kslot);
+        single_message_unit<DEC, BPT>(a, G, m, tb0, n, lane, L, kslot);
     else
-        mixed_unit<DEC, BPT>(a, G, m, starts, tb0, n, lane, L0, L1);
+        mixed_unit<DEC, BPT>(a, G, m, starts, tb0, n, lane, L);
 }
 
 // Group table staged in shared memory (read with a runtime index per tile).
@@ -214,29 +212,22 @@ __device__ __forceinline__ GroupDev load_group(uint32_t gaddr, int g) {
     return G;
 }
 
-// Units [0, E) are encryption units (groups 0-2), [E, ntiles << split) decryption
-// units.  The first enc_ctas CTAs begin with the encryption units, the others with
-// the decryption units (their numbers follow the lookups of each direction), so
-// both directions run at once and a CTA fills its tables once; one whose direction
-// has run dry swaps its tables and helps with the other, at one barrier.  Every
-// warp starts on a fixed unit of its CTA's direction (interleaved over the CTAs,
-// so a small batch spreads over the SMs), then takes units from the direction's
-// counter, independently of the other warps, so their global-memory latencies
-// overlap.  Without a counter (no direction has more units than warps) that is all.
+// Units [0, ntiles << split): encryption first (groups 0-2), then decryption; both
+// directions' tables are in shared memory throughout.  Every warp starts on a fixed
+// unit (interleaved over the CTAs, so a small batch spreads over the SMs), then
+// takes units from a counter, independently of the other warps, so their
+// global-memory latencies overlap.  Without a counter (no more units than warps)
+// that is all.
+constexpr uint32_t kBatchSlots = 2 * kTableBytes;         // key slots: 256 B per warp
+constexpr uint32_t kBatchGroups = kBatchSlots + 256u * 32;  // group table
+constexpr uint32_t kBatchSmem = kBatchGroups + 32u * kGroups;
+
 template <int BPT>
 __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const BatchArgs a) {
     pdl_trigger();
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    const uint32_t base = smem_base(smem_raw);
-    const uint32_t A = table_base(base);
-    const uint32_t gaddr = ((base + dynamic_smem_bytes()) & ~15u) - 32u * kGroups;  // group table
-    // 256 B of key slot per warp: below the 64 KiB-aligned tables when the
-    // dynamic window starts early enough, else above them.
-    const uint32_t kslots = (A >= base + 256u * 32u) ? A - 256u * 32u : A + kDecBytes;
-    if (A + kDecBytes > gaddr || (kslots >= A && kslots + 256u * 32u > gaddr)) {
-        if (threadIdx.x == 0) atomicOr(a.status, 2);
-        return;
-    }
+    const uint32_t A = smem_base(smem_raw);
+    const uint32_t gaddr = A + kBatchGroups;
 #pragma unroll
     for (int i = 0; i < kGroups; ++i) {
         if (threadIdx.x == (unsigned)i) {
@@ -247,57 +238,38 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
             for (int k = 0; k < 8; ++k) sts(gaddr + 32u * i + 4u * k, w[k]);
         }
     }
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t L0 = A | (lane << 2);
-    const uint32_t L1 = L0 | 128u;
-    const uint32_t kslot = kslots + 256u * (threadIdx.x >> 5);
-    const uint32_t warps = blockDim.x >> 5;
-    const int first_dir = blockIdx.x < a.enc_ctas ? 0 : 1;
-    fill_tables(A, first_dir != 0);
+    const uint32_t enc_tiles = a.groups[kGroups / 2 - 1].tile_end;
+    if (enc_tiles) fill_table(A, false, threadIdx.x, blockDim.x);
+    if (enc_tiles < a.ntiles) fill_table(A + kTableBytes, true, threadIdx.x, blockDim.x);
     __syncthreads();
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t L = A + 4u * lane;
+    const uint32_t kslot = A + kBatchSlots + 256u * (threadIdx.x >> 5);
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    const uint32_t units = a.ntiles << a.split;
     pdl_wait();
-    const uint32_t enc_end = lds(gaddr + 32u * 2 + 4u) << a.split;  // tile_end of group 2
-    for (int phase = 0; phase < 2; ++phase) {
-        const int dir = phase ? first_dir ^ 1 : first_dir;
-        const uint32_t u_begin = dir ? enc_end : 0u;
-        const uint32_t count = (dir ? a.ntiles << a.split : enc_end) - u_begin;
-        const uint32_t ctas = dir ? gridDim.x - a.enc_ctas : a.enc_ctas;  // CTAs that begin with this direction
-        uint32_t u;
-        if (phase == 0) {
-            u = (threadIdx.x >> 5) * ctas + (dir ? blockIdx.x - a.enc_ctas : blockIdx.x);
-        } else {
-            if (!a.counter) return;  // (every direction's units were given out at the start)
-            uint32_t left = 0;
-            if (threadIdx.x == 0) left = *(volatile unsigned*)(a.counter + dir) + ctas * warps < count;
-            if (!__syncthreads_or((int)left)) break;  // (every warp has left the other direction's units)
-            fill_tables(A, dir != 0);
-            __syncthreads();
-            u = 0;
-            if (lane == 0) u = atomicAdd(a.counter + dir, 1u) + ctas * warps;
-            u = __shfl_sync(0xffffffffu, u, 0);
-        }
-        while (u < count) {
-            uint32_t nxt = count;
-            if (a.counter && lane == 0) nxt = atomicAdd(a.counter + dir, 1u) + ctas * warps;  // consumed after this unit
-            const uint32_t t = (u + u_begin) >> a.split;
-            int g = 0;
-            while (g < kGroups - 1 && t >= lds(gaddr + 32u * g + 4u)) ++g;  // tile_end of group g
-            const GroupDev G = load_group(gaddr, g);
-            if (dir)
-                batch_warp_unit<true, BPT>(a, G, u + u_begin, lane, L0, L1, kslot);
-            else
-                batch_warp_unit<false, BPT>(a, G, u + u_begin, lane, L0, L1, kslot);
-            u = __shfl_sync(0xffffffffu, nxt, 0);
-        }
+    uint32_t u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    while (u < units) {
+        uint32_t nxt = units;
+        if (a.counter && lane == 0) nxt = atomicAdd(a.counter, 1u) + warps;  // consumed after this unit
+        const uint32_t t = u >> a.split;
+        int g = 0;
+        while (g < kGroups - 1 && t >= lds(gaddr + 32u * g + 4u)) ++g;  // tile_end of group g
+        const GroupDev G = load_group(gaddr, g);
+        if (G.dir)
+            batch_warp_unit<true, BPT>(a, G, u, lane, L + kTableBytes, kslot);
+        else
+            batch_warp_unit<false, BPT>(a, G, u, lane, L, kslot);
+        u = __shfl_sync(0xffffffffu, nxt, 0);
     }
-    // The last CTA to get here leaves the counters at zero for the next launch of
+    if (!a.counter) return;
+    // The last CTA to get here leaves the counter at zero for the next launch of
     // these tables (which waits for this one's end).
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(a.counter + kCtasDone, 1u) == gridDim.x - 1) {
             a.counter[0] = 0;
-            a.counter[1] = 0;
             a.counter[kCtasDone] = 0;
         }
     }
@@ -430,12 +402,11 @@ struct Tables {
         return img;
     }
     // Points a launch's arguments at the tables at dev.
-    void fill_args(const HostPlan& H, uint8_t* dev, int* status, BatchArgs* a) const {
+    void fill_args(const HostPlan& H, uint8_t* dev, BatchArgs* a) const {
         a->msgs = (const MsgDev*)(dev + off_msgs);
         a->keys = (const uint4*)(dev + off_keys);
         a->tile_msg = (const uint32_t*)(dev + off_tiles);
         a->counter = (unsigned*)dev;
-        a->status = status;
         a->ntiles = H.ntiles;
         a->tile_blocks = H.tile_blocks;
         memcpy(a->groups, H.groups, sizeof a->groups);
@@ -489,28 +460,10 @@ static int plan_launch_args(aes_batch_plan* P, const void* in_base, size_t in_by
     return AES_OK;
 }
 
-// The whole opt-in shared memory (the attribute is set once per kernel and context).
-static int batch_smem(BatchKernel fn, int* smem) {
-    DeviceInfo info;
-    int rc = current_device_info(&info);
-    if (rc) return rc;
-    rc = set_max_dynamic_smem((const void*)fn, info.smem_optin);
-    if (rc) return rc;
-    *smem = info.smem_optin;
-    return AES_OK;
-}
-
 // A tile is cut into the units that warps take, down to one pass of a warp,
 // until every warp has kUnitsPerWarp of them: a batch of few tiles spreads over
 // all warps, a large one keeps whole tiles (fewer unit starts).
 constexpr uint64_t kUnitsPerWarp = 4;
-
-// Up to this many blocks the two directions run side by side on CTAs of their
-// own (one table fill, one tail); above it every CTA begins with the encryption
-// tiles.  Side by side against one after the other: 50.7 / 66.1 us at 27 MB, 136.6 /
-// 150.3 at 85 MB, 400 / 408 at 291 MB, but 4,350 / 4,329 at 3.4 GB (512 x 8), where the
-// one fill and tail saved weigh less than what two streams of tiles cost.
-constexpr uint64_t kSideBySideBlocks = 1ull << 26;
 
 BatchSchedule schedule_batch(const HostPlan& H, int threads, int bpt, int sms) {
     BatchSchedule s{};
@@ -521,18 +474,7 @@ BatchSchedule schedule_batch(const HostPlan& H, int threads, int bpt, int sms) {
         ++s.split;
     const uint64_t units = (uint64_t)H.ntiles << s.split;
     s.grid = (uint32_t)std::min<uint64_t>(units, (uint64_t)sms);
-    // CTAs to each direction by its lookups (16 per block and round).
-    uint64_t work[2] = {0, 0};
-    for (const GroupDev& G : H.groups) work[G.dir] += G.blocks * (uint64_t)G.nr;
-    const uint64_t enc_units = (uint64_t)H.groups[kGroups / 2 - 1].tile_end << s.split;
-    if (work[0] && work[1] && H.total_blocks <= kSideBySideBlocks) {
-        const double share = (double)work[0] / ((double)work[0] + (double)work[1]);
-        s.enc_ctas = (uint32_t)(share * s.grid + 0.5);
-        s.enc_ctas = std::min(std::max(s.enc_ctas, 1u), s.grid - 1u);
-    } else {
-        s.enc_ctas = work[0] ? s.grid : 0u;
-    }
-    s.counted = enc_units > s.enc_ctas * warps || units - enc_units > (s.grid - s.enc_ctas) * warps;
+    s.counted = units > (uint64_t)s.grid * warps;
     return s;
 }
 
@@ -545,14 +487,12 @@ int launch_batch_kernel(const HostPlan& H, BatchArgs a, int threads, int bpt, cu
     BatchKernel fn = pick_batch(bpt);
     if (!fn) return fail(AES_ERR_ARG, "blocks_per_thread %d: need 1, 2, 4 or 8", bpt);
     if (bpt == 8 && threads > 512) return fail(AES_ERR_ARG, "8 blocks per thread need threads <= 512");
-    int smem = 0;
-    int rc = batch_smem(fn, &smem);
+    int rc = set_max_dynamic_smem((const void*)fn, (int)kBatchSmem);
     if (rc) return rc;
     const BatchSchedule sch = current_schedule(H, threads, bpt);
     a.split = sch.split;
-    a.enc_ctas = sch.enc_ctas;
     if (!sch.counted) a.counter = nullptr;
-    const cudaError_t e = launch_overlapped(fn, sch.grid, (unsigned)threads, (size_t)smem, stream, a);
+    const cudaError_t e = launch_overlapped(fn, sch.grid, (unsigned)threads, kBatchSmem, stream, a);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "batch kernel launch: %s", cudaGetErrorString(e));
     return AES_OK;
 }
@@ -627,8 +567,7 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
         return nullptr;
     }
     e = cudaMemcpy(P->dev_buf, tables.image(H, ctxs, nctx).get(), P->dev_bytes, cudaMemcpyHostToDevice);
-    int* status = nullptr;
-    if (e != cudaSuccess || device_status_word(&status)) {
+    if (e != cudaSuccess) {
         fail(AES_ERR_CUDA, "uploading the batch plan: %s", cudaGetErrorString(e));
         cudaFree(P->dev_buf);
         delete P;
@@ -636,11 +575,10 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
     }
     BatchArgs& a = P->args;
     memset(&a, 0, sizeof a);
-    tables.fill_args(H, P->dev_buf, status, &a);
+    tables.fill_args(H, P->dev_buf, &a);
     if (H.ntiles) {
         const BatchSchedule sch = current_schedule(H, P->threads, P->bpt);
         a.split = sch.split;
-        a.enc_ctas = sch.enc_ctas;
         if (!sch.counted) a.counter = nullptr;
         P->grid = sch.grid;
     }
@@ -655,10 +593,9 @@ int aes_batch_plan_launch(aes_batch_plan* P, const void* in_base, size_t in_byte
     if (rc) return rc;
     if (P->host.ntiles == 0) return AES_OK;
     BatchKernel fn = pick_batch(P->bpt);
-    int smem = 0;
-    rc = batch_smem(fn, &smem);
+    rc = set_max_dynamic_smem((const void*)fn, (int)kBatchSmem);
     if (rc) return rc;
-    const cudaError_t e = launch_overlapped(fn, P->grid, (unsigned)P->threads, (size_t)smem, (cudaStream_t)stream, a);
+    const cudaError_t e = launch_overlapped(fn, P->grid, (unsigned)P->threads, kBatchSmem, (cudaStream_t)stream, a);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "batch kernel launch: %s", cudaGetErrorString(e));
     return AES_OK;
 }
@@ -671,8 +608,7 @@ int aes_batch_plan_launch_graph(aes_batch_plan* P, const void* in_base, size_t i
     if (P->host.ntiles == 0) return AES_OK;
     std::lock_guard<std::mutex> lk(P->mu);
     BatchKernel fn = pick_batch(P->bpt);
-    int smem = 0;
-    rc = batch_smem(fn, &smem);
+    rc = set_max_dynamic_smem((const void*)fn, (int)kBatchSmem);
     if (rc) return rc;
     cudaError_t e = cudaSuccess;
     if (!P->graph_exec) {
@@ -682,7 +618,7 @@ int aes_batch_plan_launch_graph(aes_batch_plan* P, const void* in_base, size_t i
         }
         e = cudaStreamBeginCapture(P->capture_stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            fn<<<P->grid, P->threads, smem, P->capture_stream>>>(a);
+            fn<<<P->grid, P->threads, kBatchSmem, P->capture_stream>>>(a);
             e = cudaStreamEndCapture(P->capture_stream, &P->graph);
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&P->graph_exec, P->graph, 0);
@@ -708,7 +644,7 @@ int aes_batch_plan_launch_graph(aes_batch_plan* P, const void* in_base, size_t i
         kp.func = (void*)fn;
         kp.gridDim = dim3(P->grid);
         kp.blockDim = dim3(P->threads);
-        kp.sharedMemBytes = smem;
+        kp.sharedMemBytes = kBatchSmem;
         kp.kernelParams = params;
         e = cudaGraphExecKernelNodeSetParams(P->graph_exec, P->kernel_node, &kp);
         if (e != cudaSuccess) return fail(AES_ERR_CUDA, "updating the batch graph: %s", cudaGetErrorString(e));
@@ -760,8 +696,7 @@ int aes_ecb_batch(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* c
     if (e != cudaSuccess) return fail(AES_ERR_NOMEM, "cudaMallocAsync(%zu): %s", tables.bytes, cudaGetErrorString(e));
     const auto img = tables.image(H, ctxs, nctx);
     e = cudaMemcpyAsync(buf, img.get(), tables.bytes, cudaMemcpyHostToDevice, s);  // pageable: staged before return
-    int* status = nullptr;
-    if (e != cudaSuccess || device_status_word(&status)) {
+    if (e != cudaSuccess) {
         cudaFreeAsync(buf, s);
         return fail(AES_ERR_CUDA, "uploading the batch tables: %s", cudaGetErrorString(e));
     }
@@ -769,7 +704,7 @@ int aes_ecb_batch(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* c
     memset(&a, 0, sizeof a);
     a.in = (const uint4*)in_base;
     a.out = (uint4*)out_base;
-    tables.fill_args(H, buf, status, &a);
+    tables.fill_args(H, buf, &a);
     rc = launch_batch_kernel(H, a, shape.threads, shape.bpt, s);
     cudaFreeAsync(buf, s);
     return rc;
@@ -861,9 +796,6 @@ int aes_ecb_batch_noalloc(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* 
     uint8_t* buf = nullptr;
     rc = noalloc_scratch(&buf);
     if (rc) return rc;
-    int* status = nullptr;
-    rc = device_status_word(&status);
-    if (rc) return rc;
     const auto img = tables.image(H, ctxs, nctx);  // host staging only; the counter words are zero
     cudaStream_t s = (cudaStream_t)stream;
     // Stream-ordered after earlier work on `stream`; from pageable memory the
@@ -874,7 +806,7 @@ int aes_ecb_batch_noalloc(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* 
     memset(&a, 0, sizeof a);
     a.in = (const uint4*)in_base;
     a.out = (uint4*)out_base;
-    tables.fill_args(H, buf, status, &a);
+    tables.fill_args(H, buf, &a);
     return launch_batch_kernel(H, a, shape.threads, shape.bpt, s);
 }
 

@@ -28,7 +28,7 @@ struct GroupDev {
 };
 
 constexpr int kGroups = 6;
-constexpr int kCtasDone = 2;  // BatchArgs::counter[kCtasDone]
+constexpr int kCtasDone = 1;  // BatchArgs::counter[kCtasDone]
 constexpr int kSlotWords = 64;  // 60 used (Nr = 14), padded to 256 bytes
 
 struct BatchArgs {
@@ -37,13 +37,11 @@ struct BatchArgs {
     const MsgDev* msgs;
     const uint4* keys;  // kSlotWords / 4 uint4 per slot
     const uint32_t* tile_msg;
-    unsigned* counter;  // three words, zero at the launch and after it (units taken of each direction, CTAs done),
-                        // or nullptr: no direction has more units than warps
-    int* status;
+    unsigned* counter;  // two words, zero at the launch and after it (units taken, CTAs done),
+                        // or nullptr: no more units than warps
     uint32_t ntiles;
     uint32_t tile_blocks;
-    uint32_t split;     // a warp takes 1 / 2^split of a tile at a time
-    uint32_t enc_ctas;  // CTAs that begin with the encryption tiles
+    uint32_t split;  // a warp takes 1 / 2^split of a tile at a time
     GroupDev groups[kGroups];
 };
 
@@ -62,17 +60,16 @@ struct HostPlan {
 int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx, uint32_t tile_blocks,
                     HostPlan* P);
 
-// How one batched launch shares its tiles among the GPU's warps (BatchArgs::split, enc_ctas).
+// How one batched launch shares its tiles among the GPU's warps (BatchArgs::split).
 struct BatchSchedule {
     uint32_t split;
-    uint32_t enc_ctas;
     uint32_t grid;
     bool counted;  // some warps take more than one unit: the launch needs its counter, zeroed
 };
 BatchSchedule schedule_batch(const HostPlan& H, int threads, int bpt, int sms);
 
-// Launches the batched kernel (one CTA per SM at most; ntiles > 0): fills in a.split, a.enc_ctas and, where the
-// schedule needs none, clears a.counter.
+// Launches the batched kernel (one CTA per SM at most; ntiles > 0): fills in a.split and, where the schedule
+// needs none, clears a.counter.
 int launch_batch_kernel(const HostPlan& H, BatchArgs a, int threads, int bpt, cudaStream_t stream);
 
 int device_status_word(int** p);  // ecb_table.cu

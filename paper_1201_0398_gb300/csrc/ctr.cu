@@ -11,62 +11,65 @@
 // "counter-mode caching", New AES Software Speed Records, 2008; splitting round 2
 // in two parts, each common to many blocks, spares all 32 lookups of both rounds.)
 //
-// Rows of 256 counters share y.  A warp takes 32 neighbouring x of consecutive
-// rows: its lanes keep F(x, y0) ^ F(0, y0) in four registers while the upper 14
-// bytes last (2^16 counters), and F(0, y) of the next 32 rows -- the same for all
-// lanes -- in shared memory, one 16-byte broadcast load per row in place of 32
-// lookups.  Both come from two ordinary rounds, 32 lookups per lane each.
+// Rows of 256 counters share y.  A thread takes the counters x and x + 128 of
+// consecutive rows: it keeps F(x, y0) ^ F(0, y0) of both in registers while the
+// upper 14 bytes last (2^16 counters), and its warp F(0, y) of the next 32 rows --
+// the same for all lanes -- in shared memory, one 16-byte broadcast load per row in
+// place of 2 x 32 lookups.  All come from two ordinary rounds, 32 lookups per lane
+// each.
 //
 // Bound: the shared-memory lookups of the remaining Nr - 2 rounds (16 per block and
 // round, 32 lanes per clock and SM) and the L1 cycles of the global loads and
-// stores (about 16 per 32 blocks): 1 GiB of AES-128 takes 147 of the 128 + 16
-// cycles per 32 blocks, where the table kernel's ten rounds take 177.  Measured,
-// before and after: 1 GiB 908 -> 1,117 GB/s (AES-256 667 -> 771; 1,104 / 766 where the
-// input's first counter is odd, so that a warp's 512 bytes straddle five lines),
-// 256 MiB 894 -> 1,079 (658 -> 752), 16 MiB 788 -> 887 (598 -> 649).
+// stores (about 12 per 32 blocks): 1 GiB of AES-128 takes 143 of the 128 + 12
+// cycles per 32 blocks, where ten rounds take 173.  Measured, with all the rounds in
+// the table kernel and here: 1 GiB 1,153 -> 954 us (1,125 GB/s; AES-256 1,583 -> 1,382),
+// 256 MiB 291 -> 242 (400 -> 349), 16 MiB 20.6 -> 17.4 (27.0 -> 24.1).  An input whose first
+// counter is odd, so that a warp's 512 bytes straddle five lines, takes 1% more.
+// One counter a row (four rows at a time) measured 969 us at 1 GiB, four counters 947
+// (AES-256 1,433); two CTAs per SM with 64 registers a thread 984.
 #include "block_io.cuh"
 #include "launch.cuh"
-#include "rounds_dp4a.cuh"
 
 namespace gbaes {
 
-constexpr int kCtrThreads = 512;  // 8 warps span a row's 256 counters; 2 row ranges per CTA
-constexpr int kCtrHalves = kCtrThreads / 256;
-constexpr int kCtrRows = 4;         // rows a warp enciphers at a time
-constexpr uint32_t kCtrSlots = 32;  // rows whose F(0, y) a warp keeps
-constexpr uint32_t kCtrSmem = dp::kEncBytes + (kCtrThreads / 32) * kCtrSlots * 16u;
+constexpr int kCtrThreads = 512;
+constexpr int kCtrX = 2;                             // counters of a row per thread
+constexpr uint32_t kCtrSpan = 256 / kCtrX;           // threads across a row
+constexpr int kCtrRanges = kCtrThreads / kCtrSpan;   // row ranges per CTA
+constexpr uint32_t kCtrSlots = 32;                   // rows whose F(0, y) a warp keeps
+constexpr uint32_t kCtrSmem = kTableBytes + (kCtrThreads / 32) * kCtrSlots * 16u;
 
-// Rows row .. row + ROWS - 1 of this warp: v = 256 row + x is a block's counter
-// less the (2^16-aligned) counter base, and v - a.first its place in the input;
-// places outside the input (before its first counter, past its last) compute and
-// store nothing.
-template <int NR, int ROWS>
-__device__ __forceinline__ void ctr_rows(const EcbArgs& a, uint64_t row, uint32_t x, const uint32_t (&ax)[4],
-                                         uint32_t slots, uint32_t L) {
-    uint32_t s[ROWS][4];
-    uint4 data[ROWS];
+// This thread's counters of one row: v = 256 row + x + kCtrSpan * g is a block's
+// counter less the (2^16-aligned) counter base, and v - a.first its place in the
+// input; places outside the input (before its first counter, past its last) compute
+// and store nothing.
+template <int NR>
+__device__ __forceinline__ void ctr_row(const EcbArgs& a, uint64_t row, uint32_t x, const uint32_t (&ax)[kCtrX][4],
+                                        uint32_t slots, uint32_t L) {
+    uint32_t s[kCtrX][4];
+    uint4 data[kCtrX];
     const uint64_t i0 = (row << 8) + x - a.first;
 #pragma unroll
-    for (int b = 0; b < ROWS; ++b) {
-        const uint64_t i = i0 + 256u * b;
-        data[b] = i < a.nblocks ? ld_stream(a.in + i) : make_uint4(0, 0, 0, 0);
+    for (int g = 0; g < kCtrX; ++g) {
+        const uint64_t i = i0 + kCtrSpan * g;
+        data[g] = i < a.nblocks ? ld_stream(a.in + i) : make_uint4(0, 0, 0, 0);
     }
+    uint4 f;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(f.x), "=r"(f.y), "=r"(f.z), "=r"(f.w)
+                 : "r"(slots + 16u * ((uint32_t)row % kCtrSlots)));
 #pragma unroll
-    for (int b = 0; b < ROWS; ++b) {
-        uint4 f;
-        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(f.x), "=r"(f.y), "=r"(f.z), "=r"(f.w)
-                     : "r"(slots + 16u * (((uint32_t)row + b) % kCtrSlots)));
-        s[b][0] = ax[0] ^ f.x;
-        s[b][1] = ax[1] ^ f.y;
-        s[b][2] = ax[2] ^ f.z;
-        s[b][3] = ax[3] ^ f.w;
+    for (int g = 0; g < kCtrX; ++g) {
+        s[g][0] = ax[g][0] ^ f.x;
+        s[g][1] = ax[g][1] ^ f.y;
+        s[g][2] = ax[g][2] ^ f.z;
+        s[g][3] = ax[g][3] ^ f.w;
     }
-    dp::rounds_from<NR, false, 3, ROWS>(s, ParamKeys{a.rk}, L);
+    rounds_from<NR, false, 3, kCtrX, NR>(s, ParamKeys{a.rk}, L);
 #pragma unroll
-    for (int b = 0; b < ROWS; ++b) {
-        const uint64_t i = i0 + 256u * b;
-        if (i < a.nblocks) store_block<kCtr>(a, i, s[b], data[b]);
+    for (int g = 0; g < kCtrX; ++g) {
+        const uint64_t i = i0 + kCtrSpan * g;
+        if (i < a.nblocks) store_block<kCtr>(a, i, s[g], data[g]);
     }
 }
 
@@ -86,43 +89,49 @@ __device__ __forceinline__ void two_rounds(const EcbArgs& a, const uint64_t (&v)
 #pragma unroll
     for (int r = 1; r <= 2; ++r)
 #pragma unroll
-        for (int i = 0; i < N; ++i) dp::round_inner<false>(s[i], L, ks.get(r));
+        for (int i = 0; i < N; ++i) round_inner<false>(s[i], L, ks.get(r));
 }
 
 // a.ctr_hi, a.ctr_lo: the counter base, its low 16 bits 0; a.first: the first
 // block's counter less the base (below 2^16).
 template <int NR>
 __global__ void __launch_bounds__(kCtrThreads, 1) ctr_kernel(const EcbArgs a) {
-    pdl_trigger();
     extern __shared__ __align__(16) uint8_t smem_raw[];
+    pdl_trigger();
     const uint32_t A = smem_base(smem_raw);
-    dp::fill_tables<kCtrThreads, false>(A);
+    fill_table(A, false, threadIdx.x, kCtrThreads);
     __syncthreads();
     pdl_wait();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t L = A + 4u * lane;
-    const uint32_t slots = A + dp::kEncBytes + (threadIdx.x >> 5) * kCtrSlots * 16u;
-    const uint32_t x = threadIdx.x & 255u;
+    const uint32_t slots = A + kTableBytes + (threadIdx.x >> 5) * kCtrSlots * 16u;
+    const uint32_t x = threadIdx.x % kCtrSpan;
     // Rows with blocks of the input, shared out evenly over the row ranges of all CTAs.
     const uint64_t row0 = a.first >> 8;
     const uint64_t rows = ((a.first + a.nblocks - 1) >> 8) - row0 + 1;
-    const uint64_t range = (uint64_t)blockIdx.x * kCtrHalves + (threadIdx.x >> 8);
-    const uint64_t ranges = (uint64_t)gridDim.x * kCtrHalves;
+    const uint64_t range = (uint64_t)blockIdx.x * kCtrRanges + threadIdx.x / kCtrSpan;
+    const uint64_t ranges = (uint64_t)gridDim.x * kCtrRanges;
     uint64_t row = row0 + rows * range / ranges;
     const uint64_t end = row0 + rows * (range + 1) / ranges;
     uint64_t high = ~0ull;  // row / 256 that ax belongs to
-    uint32_t ax[4] = {0, 0, 0, 0};
+    uint32_t ax[kCtrX][4] = {};
     while (row < end) {
         const uint64_t slot_row = row & ~(uint64_t)(kCtrSlots - 1);
         uint32_t f[4];
         if (row >> 8 != high) {
             high = row >> 8;
-            uint32_t t[2][4];
-            two_rounds<2>(a, {(slot_row + lane) << 8, (slot_row << 8) + x}, L, t);
+            uint64_t v[kCtrX + 1];
+            uint32_t t[kCtrX + 1][4];
+            v[kCtrX] = (slot_row + lane) << 8;
+#pragma unroll
+            for (int g = 0; g < kCtrX; ++g) v[g] = (slot_row << 8) + x + kCtrSpan * g;
+            two_rounds<kCtrX + 1>(a, v, L, t);
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
-                f[w] = t[0][w];
-                ax[w] = t[1][w] ^ __shfl_sync(0xffffffffu, f[w], 0);
+                f[w] = t[kCtrX][w];
+                const uint32_t f0 = __shfl_sync(0xffffffffu, f[w], 0);
+#pragma unroll
+                for (int g = 0; g < kCtrX; ++g) ax[g][w] = t[g][w] ^ f0;
             }
         } else {
             uint32_t t[1][4];
@@ -136,8 +145,7 @@ __global__ void __launch_bounds__(kCtrThreads, 1) ctr_kernel(const EcbArgs a) {
                      : "memory");
         __syncwarp();
         const uint64_t stop = slot_row + kCtrSlots < end ? slot_row + kCtrSlots : end;
-        for (; row + kCtrRows <= stop; row += kCtrRows) ctr_rows<NR, kCtrRows>(a, row, x, ax, slots, L);
-        for (; row < stop; ++row) ctr_rows<NR, 1>(a, row, x, ax, slots, L);
+        for (; row < stop; ++row) ctr_row<NR>(a, row, x, ax, slots, L);
     }
 }
 
@@ -145,7 +153,7 @@ __global__ void __launch_bounds__(kCtrThreads, 1) ctr_kernel(const EcbArgs a) {
 // fewer the two rounds ahead of a range's first row and the uneven last rows cost
 // more than the rounds spared: 311,296 blocks (four rows) 8.28 us in the table kernel,
 // 8.47 here (AES-256 10.34 / 10.75), 400,000 blocks 10.57 / 9.85 (13.48 / 12.76).
-uint64_t ctr_min_blocks(int sms) { return (uint64_t)sms * kCtrHalves * 256u * 5u; }
+uint64_t ctr_min_blocks(int sms) { return (uint64_t)sms * 2u * 256u * 5u; }
 
 int launch_ctr(EcbArgs a, int nr, cudaStream_t stream) {
     DeviceInfo info;
@@ -154,8 +162,6 @@ int launch_ctr(EcbArgs a, int nr, cudaStream_t stream) {
     using Fn = void (*)(const EcbArgs);
     const Fn fn = nr == 10 ? ctr_kernel<10> : nr == 12 ? ctr_kernel<12> : nr == 14 ? ctr_kernel<14> : nullptr;
     if (!fn) return fail(AES_ERR_ARG, "no CTR kernel for nr=%d", nr);
-    rc = set_max_dynamic_smem((const void*)fn, kCtrSmem);
-    if (rc) return rc;
     // The first counter, split into a base with 16 zero low bits and the rest.
     const uint64_t lo = a.ctr_lo + a.first;
     if (lo < a.ctr_lo) ++a.ctr_hi;

@@ -4,74 +4,119 @@
 // 32-bit table lookups and a round-key word,
 //     O_j = T0[I_{j,0}] ^ T1[I_{j+1,1}] ^ T2[I_{j+2,2}] ^ T3[I_{j+3,3}] ^ K_j
 // (indices of I mod 4), and for the inverse cipher the same with Td tables and
-// I_{j-k,k}.  The paper keeps the tables in a texture (Section 3); here they sit
-// in shared memory in the conflict-free, one-PRMT-per-address layout described
-// in aes_rounds.cuh, 128 KiB (encryption) or 160 KiB (decryption) per CTA.
+// I_{j-k,k}.  The paper keeps the tables in a texture (Section 3); here one of them,
+// 32 times replicated, sits in shared memory (aes_rounds.cuh), the others are
+// rotations of it.
 //
-// One CTA per SM (the tables fill most of the SM's shared memory), persistent
-// over the input in tiles of threads*BPT blocks; each block is a coalesced
-// 16-byte load and store, and round keys come from the kernel parameters.
+// Two CTAs of 512 threads per SM, persistent over the input; each block is a
+// coalesced 16-byte load and store, and round keys come from the kernel parameters.
+#include <algorithm>
+
 #include "block_io.cuh"
 #include "launch.cuh"
 
 namespace gbaes {
 
-__device__ int g_status;  // nonzero: a kernel found that its shared-memory layout did not fit
+__device__ int g_status;  // nonzero: a kernel reported an error (resident.cu)
 
+// Blocks i, i + step, ... of a thread: loads, rounds and stores.  Blocks from `end`
+// on are computed on zeros and not stored.
 template <int MODE, int BPT>
-__device__ __forceinline__ void load_tile(const EcbArgs& a, uint64_t t0b, uint32_t (&s)[BPT][4], uint4 (&aux)[BPT]) {
+__device__ __forceinline__ void load_blocks(const EcbArgs& a, uint64_t i, uint32_t step, uint64_t end,
+                                            uint32_t (&s)[BPT][4], uint4 (&aux)[BPT]) {
 #pragma unroll
     for (int b = 0; b < BPT; ++b) {
-        const uint64_t idx = t0b + threadIdx.x + (uint64_t)b * blockDim.x;
-        load_block<MODE>(a, idx, idx < a.nblocks, s[b], aux[b]);
+        const uint64_t idx = i + (uint64_t)b * step;
+        load_block<MODE>(a, idx, idx < end, s[b], aux[b]);
     }
 }
 
 template <int NR, int MODE, int BPT>
+__device__ __forceinline__ void cipher_blocks(const EcbArgs& a, uint64_t i, uint32_t step, uint64_t end,
+                                              uint32_t (&s)[BPT][4], const uint4 (&aux)[BPT], uint32_t L) {
+    constexpr bool DECRYPT = (MODE == kDec || MODE == kCbcDec);
+    whiten<BPT>(s, ParamKeys{a.rk});
+    // In full: 1 GiB 1,153 us (AES-256 decryption 1,583), three rounds per iteration 1,156 (1,683).
+    rounds_from<NR, DECRYPT, 1, BPT, NR>(s, ParamKeys{a.rk}, L);
+#pragma unroll
+    for (int b = 0; b < BPT; ++b) {
+        const uint64_t idx = i + (uint64_t)b * step;
+        if (idx < end) store_block<MODE>(a, idx, s[b], aux[b]);
+    }
+}
+
+// The CTAs take passes of blockDim.x * BPT blocks in turn, as many as there are for
+// all of them, then equal shares of the rest (less than a pass each; they differ by
+// 32 blocks at most, whatever n is), one state at a time so that whole warps past
+// the end of a share skip it.  The next pass's input -- the rest's, after the last
+// full pass -- is loaded before the rounds of the pass before it, except with 4
+// blocks per thread, where holding both would spill.
+template <int NR, int MODE, int BPT>
 __global__ void __launch_bounds__(1024, 1) table_kernel(const EcbArgs a) {
     constexpr bool DECRYPT = (MODE == kDec || MODE == kCbcDec);
-    constexpr uint32_t kNeed = DECRYPT ? kDecBytes : kEncBytes;
-    pdl_trigger();  // (the next call's CTAs fit beside none of these: they start as these end)
+    constexpr bool kAhead = BPT <= 2;
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    const uint32_t base = smem_base(smem_raw);
-    const uint32_t A = table_base(base);
-    if (A + kNeed > base + dynamic_smem_bytes()) {  // same outcome in every thread of every CTA
-        if (threadIdx.x == 0) atomicOr(&g_status, 1);
-        return;
-    }
-    const uint64_t n = a.nblocks;
-    const uint64_t tile = (uint64_t)blockDim.x * BPT;
-    const uint64_t stride = (uint64_t)gridDim.x * tile;
-    uint64_t t0b = (uint64_t)blockIdx.x * tile;
-    uint32_t s[BPT][4];
-    uint4 aux[BPT];  // CTR: data; CBC: previous ciphertext block
-    fill_tables(A, DECRYPT);
+    pdl_trigger();  // (the next call's CTAs start as these end: two fill an SM's registers)
+    const uint32_t A = smem_base(smem_raw);
+    fill_table(A, DECRYPT, threadIdx.x, blockDim.x);
+    const uint32_t L = A + 4u * (threadIdx.x & 31u);
+    const uint32_t step = blockDim.x;
+    const uint64_t stride = (uint64_t)step * BPT * gridDim.x;  // blocks of one pass of every CTA
+    const uint64_t n = a.nblocks, first = n / stride * stride, units = (n - first + 31) / 32;
+    uint64_t i = (uint64_t)step * BPT * blockIdx.x + threadIdx.x;
+    uint64_t rest = first + units * blockIdx.x / gridDim.x * 32 + threadIdx.x;  // this thread's first block of the rest
+    uint64_t end = first + units * (blockIdx.x + 1) / gridDim.x * 32;
+    if (end > n) end = n;
+    uint32_t next[BPT][4];
+    uint4 next_aux[BPT];  // CTR: data; CBC: previous ciphertext block
     pdl_wait();
-    load_tile<MODE, BPT>(a, t0b, s, aux);
+    if (kAhead) {
+        const bool full = i < first;
+        load_blocks<MODE, BPT>(a, full ? i : rest, step, full ? first : end, next, next_aux);
+    }
     __syncthreads();
-
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t L0 = A | (lane << 2);
-    const uint32_t L1 = L0 | 128u;
-    // Only the last tile is partial: a thread leaves once its next block is past the end.
-    while (t0b + threadIdx.x < n) {
-        cipher<NR, DECRYPT, BPT>(s, ParamKeys{a.rk}, L0, L1);
+    while (i < first) {
+        uint32_t s[BPT][4];
+        uint4 aux[BPT];
+        const uint64_t ni = i + stride;
+        if (kAhead) {
 #pragma unroll
-        for (int b = 0; b < BPT; ++b) {
-            const uint64_t idx = t0b + threadIdx.x + (uint64_t)b * blockDim.x;
-            if (idx < n) store_block<MODE>(a, idx, s[b], aux[b]);
+            for (int b = 0; b < BPT; ++b) {
+                aux[b] = next_aux[b];
+#pragma unroll
+                for (int w = 0; w < 4; ++w) s[b][w] = next[b][w];
+            }
+            const bool full = ni < first;
+            load_blocks<MODE, BPT>(a, full ? ni : rest, step, full ? first : end, next, next_aux);
+        } else {
+            load_blocks<MODE, BPT>(a, i, step, first, s, aux);
         }
-        t0b += stride;
-        if (t0b + threadIdx.x >= n) break;
-        load_tile<MODE, BPT>(a, t0b, s, aux);
+        cipher_blocks<NR, MODE, BPT>(a, i, step, first, s, aux, L);
+        i = ni;
+    }
+#pragma unroll 1
+    for (int b = 0; b < BPT && rest < end; ++b, rest += step) {
+        uint32_t s[1][4];
+        uint4 aux[1];
+        if (kAhead) {
+            aux[0] = next_aux[0];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) s[0][w] = next[0][w];
+            next_aux[0] = next_aux[BPT - 1];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) next[0][w] = next[BPT - 1][w];
+        } else {
+            load_blocks<MODE, 1>(a, rest, step, end, s, aux);
+        }
+        cipher_blocks<NR, MODE, 1>(a, rest, step, end, s, aux, L);
     }
 }
 
 // ------------------------------------------------------------ compact tables
 //
 // Calls too small to fill the GPU are bound by latency, not by the lookup rate:
-// the 32x replicated tables (128-160 KiB per CTA) would take longer to write
-// than the few blocks each CTA enciphers.  This variant keeps each of T0..T3
+// the 32x replicated table (32 KiB per CTA) takes longer to write than the few
+// blocks each CTA enciphers.  This variant keeps each of T0..T3
 // (and the inverse S-box) once, 4-5 KiB of shared memory: one word per thread
 // to write.  Its lookups may meet bank conflicts (32 lanes, random bytes, one
 // copy), which costs little when every warp is one of a handful on its SM.
@@ -80,10 +125,12 @@ __global__ void __launch_bounds__(1024, 1) table_kernel(const EcbArgs a) {
 
 constexpr uint32_t kCompactWords = 5 * 256;
 
-// AES_KERNEL_TABLE takes the compact tables up to this many blocks per SM
-// (measured crossover on the GB300: below it the replicated tables' fill costs
-// more than the compact tables' bank conflicts).
-constexpr uint64_t kCompactBlocksPerSm = 128;
+// AES_KERNEL_TABLE takes the compact tables up to this many blocks per SM.  Measured
+// on the GB300 (AES-128 / 256 encryption, a call in a graph, compact against
+// replicated): 256 blocks 2.71 / 2.69 and 3.02 / 2.87 us, 9,728 blocks 2.63 / 3.04 and
+// 2.98 / 3.24, 13,000 blocks 3.12 / 3.17 and 3.50 / 3.44; in a stream, where fills
+// overlap the call before, 15,000 blocks 3.02 / 3.02 and 3.95 / 3.18.
+constexpr uint64_t kCompactBlocksPerSm = 64;
 
 template <int K>
 __device__ __forceinline__ uint32_t byte4(uint32_t w) {  // 4 * (byte K of w)
@@ -243,6 +290,8 @@ KernelFn pick(int nr, int mode, int bpt) {
 
 }  // namespace
 
+constexpr int kMinThreads = 128;
+
 uint64_t compact_limit_blocks(int sms) { return (uint64_t)sms * kCompactBlocksPerSm; }
 
 int launch_table(const EcbArgs& a, int nr, Mode mode, int threads, int bpt, int variant, cudaStream_t stream) {
@@ -253,6 +302,12 @@ int launch_table(const EcbArgs& a, int nr, Mode mode, int threads, int bpt, int 
     const uint64_t sms = (uint64_t)info.sms;
     if (variant == AES_KERNEL_TABLE) variant = n <= compact_limit_blocks(info.sms) ? AES_KERNEL_TABLE_COMPACT
                                                                                    : AES_KERNEL_TABLE_REPLICATED;
+    if (threads == 0 || bpt == 0) {
+        // The automatic shape: one block per thread while that covers the input, which
+        // spreads a short call over the most warps.
+        if (threads == 0) threads = 512;
+        if (bpt == 0) bpt = n <= 2 * sms * (uint64_t)threads ? 1 : 2;
+    }
     KernelFn fn = pick(nr, mode, variant == AES_KERNEL_TABLE_COMPACT ? 0 : bpt);
     if (!fn) return fail(AES_ERR_ARG, "no table kernel for nr=%d mode=%d blocks_per_thread=%d", nr, (int)mode, bpt);
     unsigned grid;
@@ -266,25 +321,15 @@ int launch_table(const EcbArgs& a, int nr, Mode mode, int threads, int bpt, int 
         grid = (unsigned)(ctas < 8 * sms ? ctas : 8 * sms);
         threads = (int)(32 * per_cta);
     } else {
-        // Dynamic shared memory: the whole opt-in limit, so the 64 KiB-aligned
-        // layout fits wherever the dynamic window starts (the kernel re-checks).
-        smem = info.smem_optin;
-        rc = set_max_dynamic_smem((const void*)fn, smem);
-        if (rc) return rc;
-        // One CTA per SM.  When each CTA takes only a few tiles, shrink the CTA so
-        // the SMs share the blocks evenly: `iters` tiles each at the given shape
-        // become `iters` tiles of just enough threads to cover n.
-        const uint64_t per_cta = (uint64_t)threads * (uint64_t)bpt;
-        const uint64_t iters = (n + sms * per_cta - 1) / (sms * per_cta);
-        if (iters <= 64) {
-            uint64_t t = (n + sms * bpt * iters - 1) / (sms * bpt * iters);
-            t = (t + 31) / 32 * 32;
-            if (t < 64) t = 64;
-            if (t < (uint64_t)threads) threads = (int)t;
-        }
-        const uint64_t tile = (uint64_t)threads * (uint64_t)bpt;
-        const uint64_t want = (n + tile - 1) / tile;
-        grid = (unsigned)(want < sms ? want : sms);
+        // Two CTAs per SM (64 registers a thread), one above 512 threads.
+        const uint64_t ctas = threads <= 512 ? 2 * sms : sms;
+        const uint64_t units = (n + 31) / 32;
+        grid = (unsigned)(units < ctas ? units : ctas);
+        // A CTA with less than one pass of blocks needs no more threads than those,
+        // but a quick fill wants some.
+        const uint64_t share = (units + grid - 1) / grid * 32;
+        if (share < (uint64_t)threads) threads = (int)(share < kMinThreads ? std::min(kMinThreads, threads) : (int)share);
+        smem = (int)kTableBytes;
     }
     const cudaError_t e = launch_overlapped(fn, grid, (unsigned)threads, (size_t)smem, stream, a);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "table kernel launch: %s", cudaGetErrorString(e));

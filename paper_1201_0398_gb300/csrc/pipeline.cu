@@ -49,10 +49,13 @@ namespace gbaes {
 
 constexpr uint32_t kPipeMagic = 0x50495045u;  // "PIPE"
 constexpr int kMaxDepth = 16;
-// Launch shape of the direct mode: 512 threads x 4 blocks per thread keeps 32 KiB
-// of loads in flight per SM, enough to cover the host link's latency.
-constexpr int kDirectThreads = 512;
-constexpr int kDirectBpt = 4;
+// Launch shape of the direct mode: one CTA of 1024 threads per SM, one block each, the
+// next pass's loads in flight during a pass's rounds.  1 / 8 / 64 / 256 MiB: 9.9 / 61 / 405 /
+// 1,585 us, against 10.1 / 62 / 436 / 1,617 with 512 x 4 (no loads ahead) and 10.1 / 70 / 417 /
+// 1,602 with two CTAs of 512 x 2: the link carries both directions best when the loads
+// of a pass are spread out over it.
+constexpr int kDirectThreads = 1024;
+constexpr int kDirectBpt = 1;
 
 static void destroy_pipeline(aes_pipeline* P) {
     for (int i = 0; i < kMaxDepth; ++i) {
@@ -145,7 +148,7 @@ int aes_pipeline_ecb(aes_pipeline* P, const aes_ctx* ctx, int decrypt, const voi
         a.nblocks = nblocks;
         return launch_table(a, ctx->nr, mode, kDirectThreads, kDirectBpt, AES_KERNEL_TABLE, user);
     }
-    int threads = 1024, bpt = 2;
+    int threads = 0, bpt = 0;
     table_default_shape(ctx->bits, decrypt, &threads, &bpt);
     std::lock_guard<std::mutex> lk(P->mu);
     cudaError_t e = cudaEventRecord(P->start, user);

@@ -5,7 +5,7 @@
 // Section 4).  The launch-per-batch server (server.cu) amortises launches over
 // micro-batches but still pays a launch, a table upload and an event per
 // batch.  In resident mode the kernel stays on the GPU instead: one CTA per SM
-// holds the shared-memory tables of one direction and takes request tiles as
+// holds both directions' shared-memory tables and takes request tiles as
 // the host publishes them into a ring in page-locked memory, which the GPU
 // reads coherently over the host link (resident.h).  A tile is the unit of
 // work: up to C * BPT consecutive blocks of one request (C compute threads),
@@ -23,8 +23,7 @@
 // serialised every claim behind one L2 atomic round trip per success: with 152
 // CTAs polling, ~38 failed swaps per claim.)  Two record slots let the
 // producer stage tile i + 1 and the compute threads start loading its input
-// while tile i is enciphered.  A CTA switches its tables to the other
-// direction when its tile is there, so every live CTA serves every request.
+// while tile i is enciphered.  Every live CTA serves every request.
 //
 // Every wait is bounded: a CTA leaves when the host sets the stop word or once
 // lifetime_ns have passed since its start (both checked by the producer
@@ -128,8 +127,7 @@ constexpr uint64_t kMaxHoldNs = 20000;
 // One poll of the producer lane (non-blocking): issues the loads of both
 // published counts, the stop word and the other direction's ticket counter
 // together (one host-link round trip).  The CTA always holds a ticket in
-// direction `dir` -- the direction its tables will be in, i.e. that of the
-// last tile it handed to its compute warps -- taken before the tile is
+// direction `dir` -- that of the last tile it handed to its compute warps -- taken before the tile is
 // published, and takes one in the other direction when that direction has
 // published tiles nobody has taken.  It hands out its own direction's tile
 // when published, unless the other direction's held tile has been published
@@ -225,7 +223,7 @@ __device__ __forceinline__ int poll_tile(const ResArgs& a, int dir, uint64_t t_s
 //   full[k]   1 arrival  (producer: slot k written)
 //   empty[k]  C/32 arrivals (every compute warp: its outputs of slot k's tile stored)
 //   free[k]   1 arrival  (completer: slot k's tile counted, the slot may be refilled)
-//   sync      C/32 arrivals (the compute warps around a table fill)
+//   sync      C/32 arrivals (the compute warps after the table fill)
 // Every wait on them is bounded by the kernel's lifetime plus kGraceNs, after
 // which the thread reports (status bit 16) and leaves; no hardware barrier is
 // used after the start, so no thread can wait on one that has left.
@@ -403,16 +401,9 @@ __device__ __forceinline__ void load_states(uint32_t sl, uint32_t tid, uint32_t 
 template <int BPT>
 __global__ void __launch_bounds__(kResidentMaxThreads + 32 * kCtlWarps, 1) resident_kernel(const ResArgs a) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    const uint32_t base = smem_base(smem_raw);
-    const uint32_t A = table_base(base);
-    const uint32_t end = (base + dynamic_smem_bytes()) & ~15u;
-    // The control block (two slots and seven mbarriers): below the tables when
-    // the dynamic window starts early enough, else above them.
-    const uint32_t ctl = (A >= base + kCtlBytes) ? A - kCtlBytes : A + kDecBytes;
-    if (A + kDecBytes > end || (ctl >= A && ctl + kCtlBytes > end)) {
-        if (threadIdx.x == 0) atomicOr(a.err, 4);
-        return;
-    }
+    const uint32_t A = smem_base(smem_raw);
+    const uint32_t ctl = A + 2 * kTableBytes;  // the control block
+    static_assert(2 * kTableBytes + kCtlBytes <= 227u * 1024, "shared memory");
     const uint32_t C = blockDim.x - 32u * kCtlWarps;  // compute threads; then the producer and completer warps
     CtlBarriers mb;
     mb.full = ctl + 2 * kSlotBytes;
@@ -442,10 +433,9 @@ __global__ void __launch_bounds__(kResidentMaxThreads + 32 * kCtlWarps, 1) resid
     }
     const uint32_t tid = threadIdx.x;
     const uint32_t lane = tid & 31u;
-    const uint32_t L0 = A | (lane << 2);
-    const uint32_t L1 = L0 | 128u;
     uint32_t sync_phase = 0;
-    fill_tables_n(A, dir != 0, tid, C);
+    fill_table(A, false, tid, C);
+    fill_table(A + kTableBytes, true, tid, C);
     if (!compute_sync(sync_mb, sync_phase, deadline)) {
         atomicOr(a.err, 16);
         return;
@@ -466,15 +456,7 @@ __global__ void __launch_bounds__(kResidentMaxThreads + 32 * kCtlWarps, 1) resid
         if (early && !leave_early) load_states<BPT>(sn_l, tid, C, sn);
         const uint4 r0 = lds_v4(sl), r2 = lds_v4(sl + 32u);
         const int tdir = (int)lds(sl + 52u);
-        if (tdir != dir) {  // swap the tables (every compute thread is done with the old ones first)
-            bool ok = compute_sync(sync_mb, sync_phase, deadline);
-            if (ok) fill_tables_n(A, tdir != 0, tid, C);
-            if (!ok || !compute_sync(sync_mb, sync_phase, deadline)) {
-                atomicOr(a.err, 16);
-                return;
-            }
-            dir = tdir;
-        }
+        const uint32_t L = A + (tdir ? kTableBytes : 0u) + 4u * lane;  // that direction's table
         uint4* out = (uint4*)(((uint64_t)r0.w << 32) | r0.z);
         const uint32_t n = r2.x, nr = r2.w;
         const OneGlobalKey keys{a.keys + (uint64_t)r2.y * 16u};
@@ -488,20 +470,20 @@ __global__ void __launch_bounds__(kResidentMaxThreads + 32 * kCtlWarps, 1) resid
             const uint32_t states = (n + C - 1) / C;  // 1..BPT, the same in every thread
             if (states <= 1) {
                 uint32_t(&s1)[1][4] = *reinterpret_cast<uint32_t(*)[1][4]>(&s[0]);
-                if (dir)
-                    cipher_rt<true, 1>(s1, keys, (int)nr, L0, L1);
+                if (tdir)
+                    cipher_rt<true, 1>(s1, keys, (int)nr, L);
                 else
-                    cipher_rt<false, 1>(s1, keys, (int)nr, L0, L1);
+                    cipher_rt<false, 1>(s1, keys, (int)nr, L);
             } else if (BPT >= 4 && states <= 2) {
                 uint32_t(&s2)[2][4] = *reinterpret_cast<uint32_t(*)[2][4]>(&s[0]);
-                if (dir)
-                    cipher_rt<true, 2>(s2, keys, (int)nr, L0, L1);
+                if (tdir)
+                    cipher_rt<true, 2>(s2, keys, (int)nr, L);
                 else
-                    cipher_rt<false, 2>(s2, keys, (int)nr, L0, L1);
-            } else if (dir) {
-                cipher_rt<true, BPT>(s, keys, (int)nr, L0, L1);
+                    cipher_rt<false, 2>(s2, keys, (int)nr, L);
+            } else if (tdir) {
+                cipher_rt<true, BPT>(s, keys, (int)nr, L);
             } else {
-                cipher_rt<false, BPT>(s, keys, (int)nr, L0, L1);
+                cipher_rt<false, BPT>(s, keys, (int)nr, L);
             }
         }
 #pragma unroll
@@ -538,6 +520,8 @@ int launch_resident(const ResArgs& a, int threads, int bpt, cudaStream_t stream)
     DeviceInfo info;
     int rc = current_device_info(&info);
     if (rc) return rc;
+    // More shared memory than the tables and the control block take: with all of it no
+    // other CTA fits beside this kernel's.
     rc = set_max_dynamic_smem((const void*)fn, info.smem_optin);
     if (rc) return rc;
     fn<<<info.sms, threads + 32 * kCtlWarps, info.smem_optin, stream>>>(a);  // + the producer and completer warps

@@ -11,7 +11,7 @@ namespace gbaes {
 // for state b; unless KS::kPerState, every state shares one key, loaded once
 // per round.
 template <bool DECRYPT, int BPT, class KS>
-__device__ __forceinline__ void cipher_rt(uint32_t (&s)[BPT][4], const KS& ks, int nr, uint32_t L0, uint32_t L1) {
+__device__ __forceinline__ void cipher_rt(uint32_t (&s)[BPT][4], const KS& ks, int nr, uint32_t L) {
     constexpr int NK = KS::kPerState ? BPT : 1;
 #pragma unroll
     for (int b = 0; b < BPT; ++b) {
@@ -27,23 +27,13 @@ __device__ __forceinline__ void cipher_rt(uint32_t (&s)[BPT][4], const KS& ks, i
 #pragma unroll
         for (int b = 0; b < NK; ++b) k[b] = ks.get(r, b);
 #pragma unroll
-        for (int b = 0; b < BPT; ++b) {
-            if (DECRYPT)
-                dec_round(s[b], L0, L1, k[b < NK ? b : 0]);
-            else
-                enc_round(s[b], L0, L1, k[b < NK ? b : 0]);
-        }
+        for (int b = 0; b < BPT; ++b) round_inner<DECRYPT>(s[b], L, k[b < NK ? b : 0]);
     }
     uint4 k[NK];
 #pragma unroll
     for (int b = 0; b < NK; ++b) k[b] = ks.get(nr, b);
 #pragma unroll
-    for (int b = 0; b < BPT; ++b) {
-        if (DECRYPT)
-            dec_last(s[b], L0, k[b < NK ? b : 0]);
-        else
-            enc_last(s[b], L0, L1, k[b < NK ? b : 0]);
-    }
+    for (int b = 0; b < BPT; ++b) round_last<DECRYPT>(s[b], L, k[b < NK ? b : 0]);
 }
 
 // Round keys staged in a shared-memory slot (16 B per round), one key for every state.

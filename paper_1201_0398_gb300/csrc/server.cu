@@ -742,7 +742,6 @@ static int launch_slot(aes_server* S, Slot& slot) {
     a.keys = S->dev_keys;
     a.tile_msg = (const uint32_t*)(slot.dev_buf + off_tiles);
     a.counter = (unsigned*)slot.dev_buf;
-    a.status = S->status;
     a.ntiles = H.ntiles;
     a.tile_blocks = H.tile_blocks;
     memcpy(a.groups, H.groups, sizeof a.groups);

@@ -157,6 +157,34 @@ def test_ctr_vs_oracle(gbaes, bits):
 
 
 @pytest.mark.parametrize("bits", BITS)
+@pytest.mark.parametrize("passes", (0, 1, 2))
+def test_full_passes_and_shares_of_the_rest(gbaes, bits, passes):
+    """The table kernel takes full passes of all CTAs, then equal shares of the rest:
+    sizes at and around whole passes of two CTAs of 512 threads per SM, a block or
+    two per thread, in every mode and, for ECB, in every launch shape that divides
+    the rest differently."""
+    rng = np.random.default_rng(bits + passes)
+    key = rng.integers(0, 256, bits // 8, dtype=np.uint8).tobytes()
+    k = gbaes.Key(key)
+    iv = rng.integers(0, 256, 16, dtype=np.uint8).tobytes()
+    base = 2 * sms() * 512
+    sizes = [max(passes, 1) * base + d for d in (-33, 0, 1, 545)] + ([2 * passes * base + 31] if passes else [257, 9728])
+    data = rng.integers(0, 256, 16 * max(sizes), dtype=np.uint8)
+    enc, dec = oracle.ecb(key, bits, data), oracle.ecb(key, bits, data, decrypt=True)
+    ctr, cbc = oracle.ctr(key, bits, iv, data), oracle.cbc_decrypt(key, bits, iv, data)
+    x = dev(data)
+    for n in sizes:
+        for threads, bpt in ((0, 0), (512, 1), (512, 2), (512, 4), (1024, 1), (96, 2), (64, 4)):
+            for d, want in ((False, enc), (True, dec)):
+                y = gbaes.ecb_ex(k, x[:16 * n], decrypt=d, kernel=gbaes.KERNEL_TABLE_REPLICATED, threads=threads,
+                                 blocks_per_thread=bpt)
+                assert np.array_equal(host(y), want[:16 * n]), (n, threads, bpt, d)
+        assert np.array_equal(host(gbaes.ctr_xcrypt(k, iv, x[:16 * n])), ctr[:16 * n]), n
+        assert np.array_equal(host(gbaes.cbc_decrypt(k, iv, x[:16 * n])), cbc[:16 * n]), n
+    assert gbaes.device_status() == 0
+
+
+@pytest.mark.parametrize("bits", BITS)
 @pytest.mark.parametrize("kind", ("CTR_BE128", "CTR_LE32_CARRY"))
 def test_ctr_long_inputs_share_their_first_rounds(gbaes, bits, kind):
     """Inputs from the length at which rows of 256 counters share the first two
