@@ -224,7 +224,6 @@ constexpr uint32_t kBatchSmem = kBatchGroups + 32u * kGroups;
 
 template <int BPT>
 __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const BatchArgs a) {
-    pdl_trigger();
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t A = smem_base(smem_raw);
     const uint32_t gaddr = A + kBatchGroups;
@@ -248,6 +247,7 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
     const uint32_t warps = gridDim.x * (blockDim.x >> 5);
     const uint32_t units = a.ntiles << a.split;
     pdl_wait();
+    pdl_trigger();  // (at the start: 136.0 us instead of 131.9 for 85 MB, 45.0 / 44.2 for 27 MB)
     uint32_t u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     while (u < units) {
         uint32_t nxt = units;
