@@ -146,7 +146,8 @@ typedef struct aes_batch_plan aes_batch_plan;
  * AES_ERR_ALIGN), groups messages by direction and key size, tiles the
  * flattened blocks (one tile = 128 * blocks_per_thread blocks, at most 512, taken
  * by one warp, or in parts by several where there are few; CTAs of `threads` threads; blocks_per_thread 1, 2, 4 or 8, with 8
- * needing threads <= 512; 0, 0 = 1024, 2) and uploads the tile table, message table and every context's two
+ * needing threads <= 512; 0, 0 = the tiles of 1024, 2, launched in the better shape
+ * for the batch's size) and uploads the tile table, message table and every context's two
  * schedules to one device allocation on the current device (cudaMalloc,
  * synchronous).  msgs and ctxs are HOST arrays, read during the call only.
  * Returns NULL on error. */
@@ -173,8 +174,8 @@ int aes_batch_plan_info(const aes_batch_plan* plan, uint64_t* total_blocks, uint
 void aes_batch_plan_free(aes_batch_plan* plan);
 
 /* One-shot batch: plan tables in stream-ordered scratch (cudaMallocAsync /
- * cudaFreeAsync on `stream`), one launch with 1024 threads x 2 blocks per
- * thread, tiles of 512 blocks (2048 for batches above 2^23 blocks).  Same arguments and rules as the plan calls.  The tables are uploaded
+ * cudaFreeAsync on `stream`), one launch in tiles of 512 blocks (2048 for
+ * batches above 2^23 blocks).  Same arguments and rules as the plan calls.  The tables are uploaded
  * from a host copy that is freed when the call returns, so a stream that is
  * being captured into a CUDA graph is refused (AES_ERR_STATE); for graphs use
  * a plan and aes_batch_plan_launch_graph. */

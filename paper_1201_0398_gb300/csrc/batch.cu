@@ -168,14 +168,12 @@ __device__ __forceinline__ void mixed_unit(const BatchArgs& a, const GroupDev& G
     }
 }
 
-// Unit u of group G: part u mod 2^split of tile u >> split (tile_blocks
+// Part `sub` of tile t of group G, `part` blocks each (a tile is tile_blocks
 // consecutive blocks of the group's block space, fewer in the group's last one).
 template <bool DEC, int BPT>
-__device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupDev& G, uint32_t u, uint32_t lane,
-                                                uint32_t L, uint32_t kslot) {
-    const uint32_t t = u >> a.split;
-    const uint32_t part = a.tile_blocks >> a.split;
-    const uint64_t tb0 = (uint64_t)(t - G.tile_start) * a.tile_blocks + (u & ((1u << a.split) - 1u)) * part;
+__device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupDev& G, uint32_t t, uint32_t sub,
+                                                uint32_t part, uint32_t lane, uint32_t L, uint32_t kslot) {
+    const uint64_t tb0 = (uint64_t)(t - G.tile_start) * a.tile_blocks + sub * part;
     if (tb0 >= G.blocks) return;
     const uint64_t left = G.blocks - tb0;
     const uint32_t n = left < part ? (uint32_t)left : part;
@@ -212,8 +210,9 @@ __device__ __forceinline__ GroupDev load_group(uint32_t gaddr, int g) {
     return G;
 }
 
-// Units [0, ntiles << split): encryption first (groups 0-2), then decryption; both
-// directions' tables are in shared memory throughout.  Every warp starts on a fixed
+// Units: the first `whole` tiles, then the others in 2^split parts each; encryption
+// first (groups 0-2), then decryption, both directions' tables in shared memory
+// throughout.  Every warp starts on a fixed
 // unit (interleaved over the CTAs, so a small batch spreads over the SMs), then
 // takes units from a counter, independently of the other warps, so their
 // global-memory latencies overlap.  Without a counter (no more units than warps)
@@ -245,21 +244,26 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
     const uint32_t L = A + 4u * lane;
     const uint32_t kslot = A + kBatchSlots + 256u * (threadIdx.x >> 5);
     const uint32_t warps = gridDim.x * (blockDim.x >> 5);
-    const uint32_t units = a.ntiles << a.split;
+    const uint32_t units = a.whole + ((a.ntiles - a.whole) << a.split);
     pdl_wait();
     pdl_trigger();  // (at the start: 136.0 us instead of 131.9 for 85 MB, 45.0 / 44.2 for 27 MB)
     uint32_t u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     while (u < units) {
         uint32_t nxt = units;
         if (a.counter && lane == 0) nxt = atomicAdd(a.counter, 1u) + warps;  // consumed after this unit
-        const uint32_t t = u >> a.split;
+        uint32_t t = u, sub = 0, part = a.tile_blocks;
+        if (u >= a.whole) {
+            t = a.whole + ((u - a.whole) >> a.split);
+            sub = (u - a.whole) & ((1u << a.split) - 1u);
+            part = a.tile_blocks >> a.split;
+        }
         int g = 0;
         while (g < kGroups - 1 && t >= lds(gaddr + 32u * g + 4u)) ++g;  // tile_end of group g
         const GroupDev G = load_group(gaddr, g);
         if (G.dir)
-            batch_warp_unit<true, BPT>(a, G, u, lane, L + kTableBytes, kslot);
+            batch_warp_unit<true, BPT>(a, G, t, sub, part, lane, L + kTableBytes, kslot);
         else
-            batch_warp_unit<false, BPT>(a, G, u, lane, L, kslot);
+            batch_warp_unit<false, BPT>(a, G, t, sub, part, lane, L, kslot);
         u = __shfl_sync(0xffffffffu, nxt, 0);
     }
     if (!a.counter) return;
@@ -460,21 +464,26 @@ static int plan_launch_args(aes_batch_plan* P, const void* in_base, size_t in_by
     return AES_OK;
 }
 
-// A tile is cut into the units that warps take, down to one pass of a warp,
-// until every warp has kUnitsPerWarp of them: a batch of few tiles spreads over
-// all warps, a large one keeps whole tiles (fewer unit starts).
-constexpr uint64_t kUnitsPerWarp = 4;
+// A batch with fewer than kTilesPerWarp tiles for every warp has its tiles cut
+// into parts, down to one pass of a warp, until there are kPartsPerWarp of them per
+// warp.  A larger one keeps whole tiles (fewer unit starts) but for the last one
+// per warp, cut the same way, so that the SMs end together: 85 MB
+// 131.0 -> 123.7 us (1024 x 2), 291 MB 399.5 -> 392.8 (512 x 8), 849 MB 1,103.4 -> 1,097.4,
+// 3.4 GB 4,293 -> 4,288.  Cutting every tile instead gives 126-129 at 85 MB and 403.6 at
+// 291 MB (1024 x 2), the unit starts costing what the even end gains.
+constexpr uint64_t kTilesPerWarp = 4;
+constexpr uint64_t kPartsPerWarp = 8;
 
 BatchSchedule schedule_batch(const HostPlan& H, int threads, int bpt, int sms) {
     BatchSchedule s{};
-    const uint64_t warps = (uint64_t)threads / 32;
+    const uint64_t warps = (uint64_t)threads / 32 * (uint64_t)sms;
     const uint32_t pass = 32u * (uint32_t)bpt;
-    while (((uint64_t)H.ntiles << s.split) < kUnitsPerWarp * warps * (uint64_t)sms &&
-           (H.tile_blocks >> s.split) % (2u * pass) == 0)
-        ++s.split;
-    const uint64_t units = (uint64_t)H.ntiles << s.split;
+    if (H.ntiles >= kTilesPerWarp * warps) s.whole = (uint32_t)(H.ntiles - warps);
+    const uint64_t cut = H.ntiles - s.whole;
+    while ((cut << s.split) < kPartsPerWarp * warps && (H.tile_blocks >> s.split) % (2u * pass) == 0) ++s.split;
+    const uint64_t units = s.whole + (cut << s.split);
     s.grid = (uint32_t)std::min<uint64_t>(units, (uint64_t)sms);
-    s.counted = units > (uint64_t)s.grid * warps;
+    s.counted = units > (uint64_t)s.grid * ((uint64_t)threads / 32);
     return s;
 }
 
@@ -490,6 +499,7 @@ int launch_batch_kernel(const HostPlan& H, BatchArgs a, int threads, int bpt, cu
     int rc = set_max_dynamic_smem((const void*)fn, (int)kBatchSmem);
     if (rc) return rc;
     const BatchSchedule sch = current_schedule(H, threads, bpt);
+    a.whole = sch.whole;
     a.split = sch.split;
     if (!sch.counted) a.counter = nullptr;
     const cudaError_t e = launch_overlapped(fn, sch.grid, (unsigned)threads, kBatchSmem, stream, a);
@@ -506,14 +516,21 @@ struct OneShot {
     int threads, bpt;
 };
 
-// 1024 x 2 at every size: 14.6 us for 2,000 messages of 16 B - 16 KiB (4.7 MB) against
-// 19.2 with 1024 x 1 and 16.6 with 512 x 8; 50.6 / 53.6 / 50.9 at 27 MB.  Above 2^23
-// blocks tiles of 512 would only lengthen the upload.
+// From this many blocks on a launch whose shape the caller left open runs 512
+// threads x 8 blocks instead of 1024 x 2: a warp reads each round's key for 8 states
+// instead of 2 (4 cycles of the L1 data stage per read, beside 16 per state), which
+// counts once unit starts and tails do not.  1024 x 2 against 512 x 8: 10.0 / 18.5 us at
+// 4.7 MB, 43.9 / 54.6 at 27 MB, 133 / 141 at 95 MB, 397 / 393 at 291 MB, 1,138 / 1,097 at 849 MB,
+// 4,464 / 4,288 at 3.4 GB.
+constexpr uint64_t kWideBlocks = 3ull << 22;
+
+// Above 2^23 blocks tiles of 512 would only lengthen the upload.
 static OneShot one_shot_shape(const aes_msg_desc* d, size_t nmsg) {
     uint64_t total = 0;
     for (size_t i = 0; d && i < nmsg; ++i) total += std::min<uint64_t>(d[i].nblocks, 1ull << 32);
     if (total <= 1u << 23) return OneShot{512, 1024, 2};
-    return OneShot{kOneShotTileMax, 1024, 2};
+    if (total < kWideBlocks) return OneShot{kOneShotTileMax, 1024, 2};
+    return OneShot{kOneShotTileMax, 512, 8};
 }
 
 }  // namespace gbaes
@@ -522,6 +539,7 @@ extern "C" {
 
 aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx,
                                       int threads, int blocks_per_thread) {
+    const bool open = threads == 0 && blocks_per_thread == 0;
     if (threads == 0) threads = 1024;
     if (blocks_per_thread == 0) blocks_per_thread = 2;
     if (threads < 64 || threads > 1024 || threads % 32) {
@@ -552,6 +570,10 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
         delete P;
         return nullptr;
     }
+    if (open && P->host.total_blocks >= kWideBlocks) {  // (the tiles stay 1024 x 2's)
+        P->threads = 512;
+        P->bpt = 8;
+    }
     if (cudaGetDevice(&P->device) != cudaSuccess) {
         fail(AES_ERR_CUDA, "no CUDA device");
         delete P;
@@ -578,6 +600,7 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
     tables.fill_args(H, P->dev_buf, &a);
     if (H.ntiles) {
         const BatchSchedule sch = current_schedule(H, P->threads, P->bpt);
+        a.whole = sch.whole;
         a.split = sch.split;
         if (!sch.counted) a.counter = nullptr;
         P->grid = sch.grid;

@@ -41,7 +41,8 @@ struct BatchArgs {
                         // or nullptr: no more units than warps
     uint32_t ntiles;
     uint32_t tile_blocks;
-    uint32_t split;  // a warp takes 1 / 2^split of a tile at a time
+    uint32_t whole;  // the first tiles, which warps take whole ...
+    uint32_t split;  // ... and of the others 1 / 2^split at a time
     GroupDev groups[kGroups];
 };
 
@@ -60,16 +61,17 @@ struct HostPlan {
 int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx, uint32_t tile_blocks,
                     HostPlan* P);
 
-// How one batched launch shares its tiles among the GPU's warps (BatchArgs::split).
+// How one batched launch shares its tiles among the GPU's warps (BatchArgs::whole, split).
 struct BatchSchedule {
+    uint32_t whole;
     uint32_t split;
     uint32_t grid;
     bool counted;  // some warps take more than one unit: the launch needs its counter, zeroed
 };
 BatchSchedule schedule_batch(const HostPlan& H, int threads, int bpt, int sms);
 
-// Launches the batched kernel (one CTA per SM at most; ntiles > 0): fills in a.split and, where the schedule
-// needs none, clears a.counter.
+// Launches the batched kernel (one CTA per SM at most; ntiles > 0): fills in a.whole and a.split and, where the
+// schedule needs none, clears a.counter.
 int launch_batch_kernel(const HostPlan& H, BatchArgs a, int threads, int bpt, cudaStream_t stream);
 
 int device_status_word(int** p);  // ecb_table.cu
