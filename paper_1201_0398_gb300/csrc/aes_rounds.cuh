@@ -55,13 +55,21 @@ __device__ __forceinline__ void sts(uint32_t addr, uint32_t v) {
     asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-// Streaming 16-byte global load that does not allocate in L1: the input is read
-// once.  Volatile, so that a load meant to go out before the rounds stays there.
+// 16-byte input loads, read once (not kept in L1) or read again soon.  Not .nc: a
+// kernel may start while the one that writes its input still runs (launch.cuh), and
+// only the coherent path is bound to see those writes after the wait.  Volatile, so
+// that a load meant to go out before the rounds stays there.
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ uint4 ld_keep(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 

@@ -506,3 +506,39 @@ def test_dependent_calls_back_to_back(gbaes, n, captured):
         want = np.concatenate(parts + [oracle.ecb(raw[2], 256, want[16 * cut:], decrypt=True)]) ^ np.uint8(i + 1)
     assert np.array_equal(host(mid), want)
     assert gbaes.device_status() == 0
+
+
+@pytest.mark.parametrize("n", (9728, 30_001, 155_649, 400_003))
+def test_dependent_calls_on_buffers_off_by_a_block(gbaes, n):
+    """Buffers that begin 16 bytes into a 32-byte sector, so that warps (and CTAs)
+    share sectors: calls that follow one another without a wait, in place and from
+    buffer to buffer, must not see a half that a cache kept from before."""
+    rng = np.random.default_rng(n)
+    raw = [rng.integers(0, 256, b // 8, dtype=np.uint8).tobytes() for b in BITS]
+    ks = [gbaes.Key(r) for r in raw]
+    iv = bytes(range(16))
+    bufs = [torch.zeros(16 * (n + 2), dtype=torch.uint8, device="cuda") for _ in range(2)]
+    x, y = (b[16:16 * (n + 1)] for b in bufs)
+    data = rng.integers(0, 256, 16 * n, dtype=np.uint8)
+    x.copy_(torch.from_numpy(data))
+    plan = gbaes.BatchPlan(gbaes.make_descs([0], [0], [n], [1], [0]), ks)
+    steps = 12
+    for i in range(steps):
+        gbaes.encrypt_ecb(ks[i % 3], x, x)
+        gbaes.cbc_decrypt(ks[(i + 1) % 3], iv, x, y)
+        gbaes.ctr_xcrypt(ks[(i + 2) % 3], iv, y, x)
+        plan.launch(x, x)
+        gbaes.decrypt_ecb(ks[i % 3], x, y)
+        gbaes.cbc_decrypt(ks[i % 3], iv, y, x)
+    want = data
+    for i in range(steps):
+        want = oracle.ecb(raw[i % 3], BITS[i % 3], want)
+        want = oracle.cbc_decrypt(raw[(i + 1) % 3], BITS[(i + 1) % 3], iv, want)
+        want = oracle.ctr(raw[(i + 2) % 3], BITS[(i + 2) % 3], iv, want)
+        want = oracle.ecb(raw[1], BITS[1], want)
+        want = oracle.ecb(raw[i % 3], BITS[i % 3], want, decrypt=True)
+        want = oracle.cbc_decrypt(raw[i % 3], BITS[i % 3], iv, want)
+    assert np.array_equal(host(x), want)
+    for b in bufs:  # nothing before or after the blocks
+        assert not host(b[:16]).any() and not host(b[16 * (n + 1):]).any()
+    assert gbaes.device_status() == 0
