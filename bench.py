@@ -121,7 +121,7 @@ def kernel_fingerprint() -> str:
     """Hash of the table kernel's device code (host launcher code excluded)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1201_0398_gb300", "csrc")
-    for name in ("ecb_table.cu", "aes_rounds.cuh", "aes_tables.h"):
+    for name in ("ecb_table.cu", "block_io.cuh", "aes_rounds.cuh", "aes_tables.h"):
         with open(os.path.join(csrc, name), "rb") as f:
             text = f.read()
         if name == "ecb_table.cu":

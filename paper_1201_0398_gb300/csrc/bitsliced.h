@@ -538,8 +538,8 @@ GBAES_HD constexpr uint32_t affine_word(uint32_t w) {
     return r;
 }
 
-// Key planes (0 or all ones) for each processing step, from a round-key
-// schedule rk (4*(nr+1) words), plane p = 8*(state byte) + bit.
+// Round keys as the bitsliced rounds add them, from a round-key schedule rk
+// (4*(nr+1) words): word c of step r, bit p of it the plane 32c + p of that step.
 // Encryption: step 0 is rk[0]; step r (1 <= r < nr) is InvMixColumns(rk[r])
 // XOR 0x63 in every byte, added to the S-box output before MixColumns
 // (MixColumns is linear and maps 0x63 in all four bytes of a column to
@@ -547,18 +547,21 @@ GBAES_HD constexpr uint32_t affine_word(uint32_t w) {
 // on A^-1 of the state, see decrypt_half): step 0 is rk[nr] XOR 0x63; step r
 // (r >= 1) is A applied to each byte of rk[nr - r], XORed with 0x63 first for
 // r < nr.
+GBAES_HD inline uint32_t key_word(const uint32_t* rk, int nr, bool decrypt, int r, int c) {
+    uint32_t w = rk[4 * (decrypt ? nr - r : r) + c];
+    if (!decrypt && r >= 1 && r < nr) w = inv_mix_word(w);
+    if (decrypt ? r < nr : r >= 1) w ^= 0x63636363u;
+    if (decrypt && r >= 1) w = affine_word(w);
+    return w;
+}
+
+// The same as planes (0 or all ones), plane p = 8*(state byte) + bit.
 GBAES_HD inline void make_key_planes(const uint32_t* rk, int nr, bool decrypt, uint32_t (*planes)[128]) {
-    for (int r = 0; r <= nr; ++r) {
-        const int src = decrypt ? nr - r : r;
-        const bool fold = decrypt ? (r < nr) : (r >= 1);
-        for (int p = 0; p < 128; ++p) {
-            uint32_t w = rk[4 * src + p / 32];
-            if (!decrypt && r >= 1 && r < nr) w = inv_mix_word(w);
-            if (fold) w ^= 0x63636363u;
-            if (decrypt && r >= 1) w = affine_word(w);
-            planes[r][p] = ((w >> (p % 32)) & 1u) ? 0xffffffffu : 0u;
+    for (int r = 0; r <= nr; ++r)
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t w = key_word(rk, nr, decrypt, r, c);
+            for (int p = 0; p < 32; ++p) planes[r][32 * c + p] = ((w >> p) & 1u) ? 0xffffffffu : 0u;
         }
-    }
 }
 
 // Lays make_key_planes' output out for HalfKeys: step r, half h, local plane q

@@ -16,8 +16,6 @@
 // staged once per CTA in shared memory, each half's row in its own banks.  The
 // kernel is bound by the integer pipe, not by shared memory: it is the measured
 // counterpart to the T-table kernel.
-#include <mutex>
-
 #include "bitsliced.h"
 #include "launch.cuh"
 #include "gbaes_internal.h"
@@ -33,7 +31,7 @@ struct BsArgs {
     const uint4* in;
     uint4* out;
     uint64_t nblocks;
-    uint32_t planes[15 * bs::kKeyStepWords];  // split_key_planes layout (8,160 bytes)
+    uint32_t keys[60];  // bs::key_word: a bit per key plane
 };
 
 // The other lane of the pair (lane ^ 1) hands over its copy of the plane.
@@ -45,7 +43,12 @@ template <int NR, bool DEC>
 __global__ void __launch_bounds__(kBsThreads, DEC ? kBsCtasPerSmDec : kBsCtasPerSmEnc)
     bitsliced_kernel(const __grid_constant__ BsArgs a) {
     __shared__ __align__(16) uint32_t keys_s[(NR + 1) * bs::kKeyStepWords];
-    for (int i = threadIdx.x; i < (NR + 1) * bs::kKeyStepWords; i += blockDim.x) keys_s[i] = a.planes[i];
+    // Key planes from the key words, in the layout of HalfKeys.  (As an 8 KB launch
+    // parameter built on the host, a plane at a time, they made a call of 4 KiB - 4 MiB take
+    // 36 us (AES-256 48); now 12-14 (16-17).)
+    for (int i = threadIdx.x; i < (NR + 1) * 128; i += blockDim.x)
+        keys_s[bs::kKeyStepWords * (i >> 7) + bs::kKeyHalfWords * ((i >> 6) & 1) + (i & 63)] =
+            0u - ((a.keys[i >> 5] >> (i & 31)) & 1u);
     __syncthreads();
     pdl_wait();
     pdl_trigger();
@@ -104,15 +107,12 @@ int launch_bitsliced(const EcbArgs& e, const uint32_t* enc_rk, int nr, Mode mode
     BsKernel fn = pick_bs(nr, dec);
     if (!fn) return fail(AES_ERR_ARG, "no bitsliced kernel for nr=%d", nr);
     (void)threads;  // the kernel's shape is fixed by its register budget: 128 threads, 4-5 CTAs per SM
-    static BsArgs a;  // 8.2 KB: built here, copied into the launch by value
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lk(mu);
+    BsArgs a{};
     a.in = e.in;
     a.out = e.out;
     a.nblocks = e.nblocks;
-    uint32_t planes[15][128];
-    bs::make_key_planes(enc_rk, nr, dec, planes);
-    bs::split_key_planes(planes, nr, a.planes);
+    for (int r = 0; r <= nr; ++r)
+        for (int c = 0; c < 4; ++c) a.keys[4 * r + c] = bs::key_word(enc_rk, nr, dec, r, c);
     DeviceInfo info;
     int rc = current_device_info(&info);
     if (rc) return rc;
