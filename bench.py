@@ -322,7 +322,7 @@ def run_e2e(g, torch, x, keys, kernel, stream, size, bytes_per_step, e2e_steps, 
     return {"value": ranks.world * e2e_steps * bytes_per_step / e2e_s / 1e9, "unit": "GB/s",
            "h2d_bytes_per_step": bytes_per_step, "d2h_bytes_per_step": bytes_per_step, "steps": e2e_steps,
            "path": "aes_pipeline_ecb, direct mode: the table kernel loads the pinned host input and stores the "
-                   "pinned host output over the host link (512 threads x 4 blocks per thread), one launch per "
+                   "pinned host output over the host link (1024 threads x 1 block per thread), one launch per "
                    "operation; one pipeline and stream per key size",
            "staged_gbs": ranks.world * e2e_steps * bytes_per_step / staged_s / 1e9,
            "staged_path": "aes_pipeline_ecb, staged mode: 64 MiB chunks over 4 device staging slots/streams "

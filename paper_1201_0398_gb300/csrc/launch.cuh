@@ -8,7 +8,7 @@
 // tables, which depend on no earlier work, and then waits (pdl_wait) for everything
 // before it in the stream to have ended and its writes to be visible.  Measured on a
 // stream of such calls, before and after: 4 KiB 4.10 -> 2.6 us (host bound), 1 MiB 6.15 ->
-// 3.07, 9 MiB 15.8 -> 12.4, 64 MiB 79.9 -> 76.6.  Filling the tables before the wait
+// 2.75, 9 MiB 15.8 -> 12.0, 64 MiB 79.9 -> 74.6.  Filling the tables before the wait
 // instead of after it is 0.7 us of that, and costs a call on its own nothing that
 // could be measured (the first block's load no longer overlaps the fill).
 //
