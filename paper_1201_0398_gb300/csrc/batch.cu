@@ -12,11 +12,11 @@
 //    gets a slot holding its 4*(Nr+1)-word schedule.  Everything sits in one
 //    device buffer, uploaded once per plan.
 //  * Kernel.  One CTA per SM holds both directions' tables (aes_rounds.cuh).
-//    Each *warp* starts on a fixed unit (a tile, or a part of one where there are
-//    fewer tiles than warps to share them), then takes units from an atomic
+//    Each *warp* starts on a fixed unit (a few tiles, or a part of one where there are
+//    few tiles for the warps to share), then takes units from an atomic
 //    counter on its own, so the dependent loads at the start of one warp's unit
-//    overlap the other warps' lookups.  A warp whose unit lies in one message stages that
-//    message's schedule in its shared-memory key slot; in other units every block
+//    overlap the other warps' lookups.  Where its blocks lie in one message a warp stages
+//    that message's schedule in its shared-memory key slot; elsewhere every block
 //    finds its message from the starts of the next 32, and keys come from
 //    global memory through L1.  The round count is a run-time loop bound,
 //    so one compact body per direction serves all key sizes.
@@ -86,7 +86,7 @@ __device__ __forceinline__ void single_message_unit(const BatchArgs& a, const Gr
             s[b][2] = v.z;
             s[b][3] = v.w;
         }
-        if (it == 0) {  // (every lane has left the previous unit: the warp met at the unit-index shuffle)
+        if (it == 0) {  // (every lane is done with the slot: the warp met to choose these blocks)
             if (lane < (uint32_t)G.nr + 1u) {
                 const uint4 k = __ldg(a.keys + (uint64_t)q1.z * (kSlotWords / 4) + lane);
                 asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(kslot + 16u * lane), "r"(k.x),
@@ -104,12 +104,13 @@ __device__ __forceinline__ void single_message_unit(const BatchArgs& a, const Gr
     }
 }
 
-// n consecutive blocks from tb0 that cross message boundaries, the first of them
-// in message m; `starts`: load_starts of a message at most 32 before the next
-// boundary.  Each block finds its message from the window of starts: a ballot
-// counts those a pass leaves behind, an OR over the warp marks the blocks at which
-// a message begins, and a lane's message is the one of block 0 plus the marks up
-// to the lane.  (A binary search per block took five or more dependent loads;
+// The passes (32*BPT blocks) from tb0 + it on up to tb0 + end, in a unit that ends at
+// tb0 + n and crosses message boundaries; block `it` is in message m; `starts`:
+// load_starts of a message at most 32 before the next boundary.  Both are left as
+// the block after the last pass needs them.  Each block finds its message from the
+// window of starts: a ballot counts those a pass leaves behind, an OR over the warp
+// marks the blocks at which a message begins, and a lane's message is the one of
+// block 0 plus the marks up to the lane.  (A binary search per block took five or more dependent loads;
 // with the finer units of schedule_batch, the kernel's time for 2,000 messages of
 // 16 B - 16 KiB went from 33 to 14 us in a plan of 1024 x 2 and from 199 to 15 us in
 // a one-shot call.)  The states of one thread may belong to different messages:
@@ -117,10 +118,11 @@ __device__ __forceinline__ void single_message_unit(const BatchArgs& a, const Gr
 // schedule's second line is fetched ahead, and the warp runs one interleaved
 // cipher over all of them (no divergent per-block ciphers at a boundary).
 template <bool DEC, int BPT>
-__device__ __forceinline__ void mixed_unit(const BatchArgs& a, const GroupDev& G, uint32_t m, uint32_t starts,
-                                           uint64_t tb0, uint32_t n, uint32_t lane, uint32_t L) {
+__device__ __forceinline__ void mixed_passes(const BatchArgs& a, const GroupDev& G, uint32_t& m, uint32_t& starts,
+                                             uint64_t tb0, uint32_t it, uint32_t end, uint32_t n, uint32_t lane,
+                                             uint32_t L) {
     uint32_t wlast = __shfl_sync(0xffffffffu, starts, 31);  // the window's last entry
-    for (uint32_t it = 0; it < n; it += 32u * BPT) {
+    for (; it < end; it += 32u * BPT) {
         uint32_t s[BPT][4];
         uint64_t oidx[BPT];
         uint32_t slot[BPT];
@@ -168,17 +170,18 @@ __device__ __forceinline__ void mixed_unit(const BatchArgs& a, const GroupDev& G
     }
 }
 
-// Part `sub` of tile t of group G, `part` blocks each (a tile is tile_blocks
-// consecutive blocks of the group's block space, fewer in the group's last one).
-template <bool DEC, int BPT>
-__device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupDev& G, uint32_t t, uint32_t sub,
-                                                uint32_t part, uint32_t lane, uint32_t L, uint32_t kslot) {
+// The tiles [t, e) of group G, or part `sub` of tile t, `part` blocks in all (a tile is
+// tile_blocks consecutive blocks of the group's block space, fewer in the group's last one).
+template <bool DEC, int BPT, bool JOINED>
+__device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupDev& G, uint32_t t, uint32_t e,
+                                                uint32_t sub, uint32_t part, uint32_t lane, uint32_t L,
+                                                uint32_t kslot) {
     const uint64_t tb0 = (uint64_t)(t - G.tile_start) * a.tile_blocks + sub * part;
     if (tb0 >= G.blocks) return;
     const uint64_t left = G.blocks - tb0;
     const uint32_t n = left < part ? (uint32_t)left : part;
     const uint32_t m_lo = a.tile_msg[t];
-    const uint32_t m_hi = (t + 1 < G.tile_end) ? a.tile_msg[t + 1] : G.msg_end - 1;
+    const uint32_t m_hi = e < G.tile_end ? a.tile_msg[e] : G.msg_end - 1;
     uint32_t m = m_lo, starts = kNoBoundary;
     if (m_lo != m_hi) {
         for (;;) {  // find tb0's message; the starts after it stay in the window
@@ -188,10 +191,35 @@ __device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupD
             if (passed < 32u) break;
         }
     }
-    if (!__any_sync(0xffffffffu, starts != 0u && starts < n))
-        single_message_unit<DEC, BPT>(a, G, m, tb0, n, lane, L, kslot);
-    else
-        mixed_unit<DEC, BPT>(a, G, m, starts, tb0, n, lane, L);
+    constexpr uint32_t kPass = 32u * BPT;
+    const bool crossing = __any_sync(0xffffffffu, starts != 0u && starts < n);
+    if (!JOINED) {
+        if (!crossing)
+            single_message_unit<DEC, BPT>(a, G, m, tb0, n, lane, L, kslot);
+        else
+            mixed_passes<DEC, BPT>(a, G, m, starts, tb0, 0, n, n, lane, L);
+        return;
+    }
+    // Whole passes up to the next message's start (or the end) run with one message's
+    // keys, those that cross a start one by one.
+    uint32_t len = crossing ? 0u : n;
+    for (uint32_t it = 0; it < n;) {
+        uint32_t next = 0;
+        if (len == 0u) {
+            if (__shfl_sync(0xffffffffu, starts, 31) <= it) starts = load_starts(a, G, m, tb0, lane);
+            next = __reduce_min_sync(0xffffffffu, starts > it ? starts : kNoBoundary);
+            len = next >= n ? n - it : (next - it) & ~(kPass - 1u);
+        }
+        if (len) {
+            single_message_unit<DEC, BPT>(a, G, m, tb0 + it, len, lane, L, kslot);
+            it += len;
+            m += next == it;
+            len = 0;
+        } else {
+            mixed_passes<DEC, BPT>(a, G, m, starts, tb0, it, it + 1, n, lane, L);
+            it += kPass;
+        }
+    }
 }
 
 // Group table staged in shared memory (read with a runtime index per tile).
@@ -210,18 +238,18 @@ __device__ __forceinline__ GroupDev load_group(uint32_t gaddr, int g) {
     return G;
 }
 
-// Units: the first `whole` tiles, then the others in 2^split parts each; encryption
-// first (groups 0-2), then decryption, both directions' tables in shared memory
-// throughout.  Every warp starts on a fixed
-// unit (interleaved over the CTAs, so a small batch spreads over the SMs), then
-// takes units from a counter, independently of the other warps, so their
-// global-memory latencies overlap.  Without a counter (no more units than warps)
-// that is all.
+// Units: the first `whole` tiles, 2^join of them each (JOINED; a unit that reaches into
+// another group takes its tiles group by group), then the others in 2^split parts
+// each; encryption first (groups 0-2), then decryption, both directions' tables in
+// shared memory throughout.  Every warp starts on a fixed unit (interleaved over the
+// CTAs, so a small batch spreads over the SMs), then takes units from a counter,
+// independently of the other warps, so their global-memory latencies overlap.
+// Without a counter (no more units than warps) that is all.
 constexpr uint32_t kBatchSlots = 2 * kTableBytes;         // key slots: 256 B per warp
 constexpr uint32_t kBatchGroups = kBatchSlots + 256u * 32;  // group table
 constexpr uint32_t kBatchSmem = kBatchGroups + 32u * kGroups;
 
-template <int BPT>
+template <int BPT, bool JOINED>
 __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const BatchArgs a) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t A = smem_base(smem_raw);
@@ -244,26 +272,36 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
     const uint32_t L = A + 4u * lane;
     const uint32_t kslot = A + kBatchSlots + 256u * (threadIdx.x >> 5);
     const uint32_t warps = gridDim.x * (blockDim.x >> 5);
-    const uint32_t units = a.whole + ((a.ntiles - a.whole) << a.split);
+    const uint32_t units = (a.whole >> a.join) + ((a.ntiles - a.whole) << a.split);
     pdl_wait();
     pdl_trigger();  // (at the start: 136.0 us instead of 131.9 for 85 MB, 45.0 / 44.2 for 27 MB)
     uint32_t u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     while (u < units) {
         uint32_t nxt = units;
         if (a.counter && lane == 0) nxt = atomicAdd(a.counter, 1u) + warps;  // consumed after this unit
-        uint32_t t = u, sub = 0, part = a.tile_blocks;
-        if (u >= a.whole) {
-            t = a.whole + ((u - a.whole) >> a.split);
-            sub = (u - a.whole) & ((1u << a.split) - 1u);
+        const uint32_t join = JOINED ? a.join : 0u;
+        uint32_t t = u << join, end = t + (1u << join), sub = 0, part = a.tile_blocks;
+        if (t >= a.whole) {
+            const uint32_t c = u - (a.whole >> join);
+            t = a.whole + (c >> a.split);
+            end = t + 1;
+            sub = c & ((1u << a.split) - 1u);
             part = a.tile_blocks >> a.split;
         }
-        int g = 0;
-        while (g < kGroups - 1 && t >= lds(gaddr + 32u * g + 4u)) ++g;  // tile_end of group g
-        const GroupDev G = load_group(gaddr, g);
-        if (G.dir)
-            batch_warp_unit<true, BPT>(a, G, t, sub, part, lane, L + kTableBytes, kslot);
-        else
-            batch_warp_unit<false, BPT>(a, G, t, sub, part, lane, L, kslot);
+        do {
+            int g = 0;
+            while (g < kGroups - 1 && t >= lds(gaddr + 32u * g + 4u)) ++g;  // tile_end of group g
+            const GroupDev G = load_group(gaddr, g);
+            const uint32_t e = JOINED && end > G.tile_end ? G.tile_end : end;
+            if (JOINED) part *= e - t;
+            if (G.dir)
+                batch_warp_unit<true, BPT, JOINED>(a, G, t, e, sub, part, lane, L + kTableBytes, kslot);
+            else
+                batch_warp_unit<false, BPT, JOINED>(a, G, t, e, sub, part, lane, L, kslot);
+            if (!JOINED) break;
+            t = e;
+            part = a.tile_blocks;
+        } while (t < end);
         u = __shfl_sync(0xffffffffu, nxt, 0);
     }
     if (!a.counter) return;
@@ -366,6 +404,7 @@ struct aes_batch_plan {
     size_t dev_bytes;
     BatchArgs args;  // device pointers and schedule filled in; in/out set per launch
     uint32_t grid;
+    bool joined;
     cudaGraphExec_t graph_exec;
     cudaGraph_t graph;
     cudaGraphNode_t kernel_node;
@@ -425,12 +464,12 @@ struct Tables {
 
 using BatchKernel = void (*)(const BatchArgs);
 
-static BatchKernel pick_batch(int bpt) {
+static BatchKernel pick_batch(int bpt, bool joined = false) {
     switch (bpt) {
-        case 1: return batch_kernel<1>;
-        case 2: return batch_kernel<2>;
-        case 4: return batch_kernel<4>;
-        case 8: return batch_kernel<8>;  // (512 threads at most: 128 registers per thread)
+        case 1: return batch_kernel<1, false>;
+        case 2: return joined ? batch_kernel<2, true> : batch_kernel<2, false>;
+        case 4: return batch_kernel<4, false>;
+        case 8: return joined ? batch_kernel<8, true> : batch_kernel<8, false>;  // (512 threads at most: 128 registers)
         default: return nullptr;
     }
 }
@@ -466,22 +505,50 @@ static int plan_launch_args(aes_batch_plan* P, const void* in_base, size_t in_by
 
 // A batch with fewer than kTilesPerWarp tiles for every warp has its tiles cut
 // into parts, down to one pass of a warp, until there are kPartsPerWarp of them per
-// warp.  A larger one keeps whole tiles (fewer unit starts) but for the last one
-// per warp, cut the same way, so that the SMs end together: 85 MB
+// warp.  A larger one keeps whole tiles (fewer unit starts) but for the last ones
+// of every warp, cut the same way, so that the SMs end together: 85 MB
 // 131.0 -> 123.7 us (1024 x 2), 291 MB 399.5 -> 392.8 (512 x 8), 849 MB 1,103.4 -> 1,097.4,
 // 3.4 GB 4,293 -> 4,288.  Cutting every tile instead gives 126-129 at 85 MB and 403.6 at
 // 291 MB (1024 x 2), the unit starts costing what the even end gains.
+//
+// Whole tiles are then taken 2^join at a time, as long as that leaves kTilesPerWarp
+// units per warp, up to kJoinMax blocks and a kJoinPerMsg-th of the mean message
+// (messages up to 4 MiB, 512 x 8: 3.37 GB 4,285 us with tiles of 512 blocks one at a
+// time, 4,246 with 1,024 blocks, 4,234 with 2,048, 4,230 with 4,096; 10,000 messages up
+// to 256 KiB, 1,700 blocks on average, 271 MB: 382 with 512, 398 with 1,024, 455 with 2,048).
 constexpr uint64_t kTilesPerWarp = 4;
 constexpr uint64_t kPartsPerWarp = 8;
+constexpr uint64_t kJoinMax = 2048;  // blocks
+constexpr uint64_t kJoinPerMsg = 4;
+
+// The kernel for whole tiles runs each pass of a unit by itself: in a unit that
+// messages start in, the passes without a start keep to one message's keys.  It pays
+// where units have several passes: 512 x 8, 10,000 messages up to 128 KiB (146 MB)
+// 259 -> 242 us, up to 256 KiB 398 -> 382, up to 1 MiB 1,234 -> 1,218.  With 2 blocks
+// per thread (146 MB: 207.0 -> 204.6) it costs 0.6% where few units cross (250
+// messages up to 4 MiB, 92 MB: 128.1 -> 128.9), so there it wants joined tiles or a
+// mean message below kShortTiles tiles; with 4 it would spill.  In launches of cut
+// tiles it costs 0.5-4%.
+constexpr uint64_t kShortTiles = 16;
 
 BatchSchedule schedule_batch(const HostPlan& H, int threads, int bpt, int sms) {
     BatchSchedule s{};
     const uint64_t warps = (uint64_t)threads / 32 * (uint64_t)sms;
     const uint32_t pass = 32u * (uint32_t)bpt;
-    if (H.ntiles >= kTilesPerWarp * warps) s.whole = (uint32_t)(H.ntiles - warps);
+    if (H.ntiles >= kTilesPerWarp * warps) {
+        if (bpt == 2 || bpt == 8) {
+            const uint64_t mean = H.total_blocks / H.msgs.size(), most = std::min(kJoinMax, mean / kJoinPerMsg);
+            while (H.ntiles >= (kTilesPerWarp * warps << (s.join + 1)) && H.ntiles < 1u << 30 &&
+                   (uint64_t)H.tile_blocks << (s.join + 1) <= most)
+                ++s.join;
+            s.joined = (uint64_t)H.tile_blocks << s.join > pass &&
+                       (bpt == 8 || s.join || mean < kShortTiles * H.tile_blocks);
+        }
+        s.whole = (uint32_t)(H.ntiles - (warps << s.join)) >> s.join << s.join;
+    }
     const uint64_t cut = H.ntiles - s.whole;
     while ((cut << s.split) < kPartsPerWarp * warps && (H.tile_blocks >> s.split) % (2u * pass) == 0) ++s.split;
-    const uint64_t units = s.whole + (cut << s.split);
+    const uint64_t units = (s.whole >> s.join) + (cut << s.split);
     s.grid = (uint32_t)std::min<uint64_t>(units, (uint64_t)sms);
     s.counted = units > (uint64_t)s.grid * ((uint64_t)threads / 32);
     return s;
@@ -493,13 +560,14 @@ static BatchSchedule current_schedule(const HostPlan& H, int threads, int bpt) {
 }
 
 int launch_batch_kernel(const HostPlan& H, BatchArgs a, int threads, int bpt, cudaStream_t stream) {
-    BatchKernel fn = pick_batch(bpt);
-    if (!fn) return fail(AES_ERR_ARG, "blocks_per_thread %d: need 1, 2, 4 or 8", bpt);
+    if (!pick_batch(bpt)) return fail(AES_ERR_ARG, "blocks_per_thread %d: need 1, 2, 4 or 8", bpt);
     if (bpt == 8 && threads > 512) return fail(AES_ERR_ARG, "8 blocks per thread need threads <= 512");
+    const BatchSchedule sch = current_schedule(H, threads, bpt);
+    const BatchKernel fn = pick_batch(bpt, sch.joined);
     int rc = set_max_dynamic_smem((const void*)fn, (int)kBatchSmem);
     if (rc) return rc;
-    const BatchSchedule sch = current_schedule(H, threads, bpt);
     a.whole = sch.whole;
+    a.join = sch.join;
     a.split = sch.split;
     if (!sch.counted) a.counter = nullptr;
     const cudaError_t e = launch_overlapped(fn, sch.grid, (unsigned)threads, kBatchSmem, stream, a);
@@ -519,9 +587,10 @@ struct OneShot {
 // From this many blocks on a launch whose shape the caller left open runs 512
 // threads x 8 blocks instead of 1024 x 2: a warp reads each round's key for 8 states
 // instead of 2 (4 cycles of the L1 data stage per read, beside 16 per state), which
-// counts once unit starts and tails do not.  1024 x 2 against 512 x 8: 10.0 / 18.5 us at
-// 4.7 MB, 43.9 / 54.6 at 27 MB, 133 / 141 at 95 MB, 397 / 393 at 291 MB, 1,138 / 1,097 at 849 MB,
-// 4,464 / 4,288 at 3.4 GB.
+// counts once unit starts and tails do not.  1024 x 2 against 512 x 8, messages up to
+// 4 MiB: 42.5 / 44.7 us at 24 MB, 124 / 124 at 89 MB, 213 / 210 at 149 MB, 315 / 305 at
+// 231 MB, 397 / 384 at 294 MB, 1,218 / 1,175 at 918 MB, 4,395 / 4,235 at 3.4 GB; shorter
+// messages: 205 / 242 at 146 MB (up to 128 KiB), 10.3 / 19.0 at 4.7 MB (up to 16 KiB).
 constexpr uint64_t kWideBlocks = 3ull << 22;
 
 // Above 2^23 blocks tiles of 512 would only lengthen the upload.
@@ -601,9 +670,11 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
     if (H.ntiles) {
         const BatchSchedule sch = current_schedule(H, P->threads, P->bpt);
         a.whole = sch.whole;
+        a.join = sch.join;
         a.split = sch.split;
         if (!sch.counted) a.counter = nullptr;
         P->grid = sch.grid;
+        P->joined = sch.joined;
     }
     P->magic = kPlanMagic;
     return P;
@@ -615,7 +686,7 @@ int aes_batch_plan_launch(aes_batch_plan* P, const void* in_base, size_t in_byte
     int rc = plan_launch_args(P, in_base, in_bytes, out_base, out_bytes, &a);
     if (rc) return rc;
     if (P->host.ntiles == 0) return AES_OK;
-    BatchKernel fn = pick_batch(P->bpt);
+    BatchKernel fn = pick_batch(P->bpt, P->joined);
     rc = set_max_dynamic_smem((const void*)fn, (int)kBatchSmem);
     if (rc) return rc;
     const cudaError_t e = launch_overlapped(fn, P->grid, (unsigned)P->threads, kBatchSmem, (cudaStream_t)stream, a);
@@ -630,7 +701,7 @@ int aes_batch_plan_launch_graph(aes_batch_plan* P, const void* in_base, size_t i
     if (rc) return rc;
     if (P->host.ntiles == 0) return AES_OK;
     std::lock_guard<std::mutex> lk(P->mu);
-    BatchKernel fn = pick_batch(P->bpt);
+    BatchKernel fn = pick_batch(P->bpt, P->joined);
     rc = set_max_dynamic_smem((const void*)fn, (int)kBatchSmem);
     if (rc) return rc;
     cudaError_t e = cudaSuccess;

@@ -41,8 +41,9 @@ struct BatchArgs {
                         // or nullptr: no more units than warps
     uint32_t ntiles;
     uint32_t tile_blocks;
-    uint32_t whole;  // the first tiles, which warps take whole ...
-    uint32_t split;  // ... and of the others 1 / 2^split at a time
+    uint32_t whole;  // the first tiles, which warps take 2^join at a time ...
+    uint32_t join;
+    uint32_t split;  // ... and of the others 1 / 2^split of one
     GroupDev groups[kGroups];
 };
 
@@ -64,6 +65,8 @@ int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ct
 // How one batched launch shares its tiles among the GPU's warps (BatchArgs::whole, split).
 struct BatchSchedule {
     uint32_t whole;
+    uint32_t join;
+    bool joined;  // whole units have several passes: the kernel that runs each by itself
     uint32_t split;
     uint32_t grid;
     bool counted;  // some warps take more than one unit: the launch needs its counter, zeroed

@@ -172,6 +172,32 @@ def test_batch_message_boundaries(gbaes, lengths, threads, bpt, directions):
     assert gbaes.device_status() == 0
 
 
+# A launch with four tiles or more for every warp takes whole tiles, up to 2,048 blocks of them at a time where
+# messages are long, and runs the passes that no message starts in with one message's keys.
+@pytest.mark.gpu
+@pytest.mark.parametrize("threads,bpt", [(64, 2), (64, 8)])
+@pytest.mark.parametrize("longest,total", [(900, 700_000), (8200, 1_300_000), (60_000, 3_200_000)])
+def test_batch_whole_tiles_at_a_time(gbaes, threads, bpt, longest, total):
+    rng = np.random.default_rng(total)
+    nblocks = rng.integers(1, longest + 1, 2 * total // longest + 64)
+    nblocks[::17] = 1
+    nblocks[5::40] = 2048
+    n = len(nblocks)
+    ks = [gbaes.Key(rng.integers(0, 256, b // 8, dtype=np.uint8).tobytes()) for b in (128, 192, 256) * 20]
+    key_index, decrypt = rng.integers(0, len(ks), n), rng.integers(0, 2, n)
+    off = (np.cumsum(nblocks) - nblocks) * 16
+    x = torch.randint(0, 256, (16 * int(nblocks.sum()),), dtype=torch.uint8, device="cuda")
+    want, y = torch.zeros_like(x), torch.zeros_like(x)
+    for i in range(n):
+        a, b = int(off[i]), int(off[i] + 16 * nblocks[i])
+        (gbaes.decrypt_ecb if decrypt[i] else gbaes.encrypt_ecb)(ks[key_index[i]], x[a:b], want[a:b])
+    plan = gbaes.BatchPlan(gbaes.make_descs(off, off, nblocks, key_index, decrypt), ks, threads, bpt)
+    for graph in (False, True, False):
+        y.zero_()
+        plan.launch(x, y, graph=graph)
+        assert torch.equal(y, want)
+
+
 @pytest.mark.gpu
 def test_batch_graph_rebase_one_shot_and_in_place(gbaes):
     rng = np.random.default_rng(42)
