@@ -725,9 +725,9 @@ static int launch_slot(aes_server* S, Slot& slot) {
     // (schedule_batch), so a small batch keeps its latency and a large one gets no table
     // of thousands of tiles: with tiles of one pass, 256 requests of 64 B - 1 MiB (27 MB)
     // took 205 us from launch to completion, most of it building and uploading 57,000
-    // entries and reading one per 32 blocks; now 81 us.  At 200k requests/s (two per
-    // batch) p50 / p99 went from 32.9 / 54.3 to 26.3 / 41.6 us, at 800k from 56.0 / 101.5
-    // to 35.5 / 54.9.
+    // entries and reading one per 32 blocks; 81 us with these, 65 with the wide shape
+    // below.  At 200k requests/s (two per batch) p50 / p99 went from 32.9 / 54.3 to
+    // 25 / 39 us, at 800k from 56.0 / 101.5 to 31 / 48.
     const uint32_t tb = kServerTileBlocks;
     int rc = build_host_plan(d.data(), d.size(), S->key_ptrs.data(), S->key_ptrs.size(), tb, &H);
     if (rc) return rc;
