@@ -319,6 +319,8 @@ __global__ void __launch_bounds__(BPT == 8 ? 512 : 1024, 1) batch_kernel(const B
 
 // ------------------------------------------------------------------ host plan
 
+constexpr size_t kMaxMessages = 0xFFFFFFF0u;
+
 static int group_of(int nr, int dir) { return dir * 3 + (nr == 10 ? 0 : nr == 12 ? 1 : 2); }
 
 // Validates the descriptors and lays out groups and tiles: one pass checks and
@@ -327,7 +329,7 @@ int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ct
                     HostPlan* P) {
     if (nmsg && !d) return fail(AES_ERR_ARG, "message descriptors are NULL");
     if (nctx && !ctxs) return fail(AES_ERR_ARG, "key contexts are NULL");
-    if (nmsg > 0xFFFFFFF0u) return fail(AES_ERR_ARG, "too many messages (%zu)", nmsg);
+    if (nmsg > kMaxMessages) return fail(AES_ERR_ARG, "too many messages (%zu)", nmsg);
     if (tile_blocks == 0) return fail(AES_ERR_ARG, "tile size is zero");
     for (size_t i = 0; i < nctx; ++i)
         if (!ctxs[i] || ctxs[i]->magic != kCtxMagic) return fail(AES_ERR_ARG, "ctxs[%zu] is not a valid aes_ctx", i);
@@ -596,6 +598,7 @@ constexpr uint64_t kWideBlocks = 3ull << 22;
 // Above 2^23 blocks tiles of 512 would only lengthen the upload.
 static OneShot one_shot_shape(const aes_msg_desc* d, size_t nmsg) {
     uint64_t total = 0;
+    if (nmsg > kMaxMessages) nmsg = 0;  // (build_host_plan refuses the count before it reads a message)
     for (size_t i = 0; d && i < nmsg; ++i) total += std::min<uint64_t>(d[i].nblocks, 1ull << 32);
     if (total <= 1u << 23) return OneShot{512, 1024, 2};
     if (total < kWideBlocks) return OneShot{kOneShotTileMax, 1024, 2};

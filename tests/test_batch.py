@@ -3,6 +3,10 @@
 Every message of a batch must come out exactly as the CPU oracle computes it
 and exactly as the single-message kernel computes it alone (AES output is
 unique, so "the same alone and in the mix" is bit equality)."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -77,6 +81,37 @@ def test_batch_descriptor_errors(gbaes):
     with pytest.raises(gbaes.AesError):
         gbaes.batch_tiles(overflow, ks, 64)
     assert gbaes.batch_tiles(gbaes.make_descs([], [], [], [], []), ks, 64).size == 0
+
+
+# Run in a process of its own, which the two calls below took down once: {limit} is the address space it may
+# add to what it holds when the library is loaded, in bytes.
+REFUSED = """
+import ctypes, resource, sys
+import paper_1201_0398_gb300 as g
+lib, k = g.load(), g.Key(bytes(16))
+ctxs = (ctypes.c_void_p * 1)(k.handle.value)
+d = g.make_descs([0], [0], [1], [{key}], [0])
+msgs, big = ctypes.c_void_p(d.ctypes.data), ctypes.c_void_p(1 << 20)
+if {limit}:
+    held = 4096 * int(open("/proc/self/statm").read().split()[0])
+    resource.setrlimit(resource.RLIMIT_AS, (held + {limit}, held + {limit}))
+rc = {call}
+print(rc, lib.aes_last_error().decode())
+"""
+
+
+def refused(call, key=0, limit=0):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", REFUSED.format(call=call, key=key, limit=limit)], cwd=root,
+                       capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stderr)
+    return r.stdout
+
+
+def test_message_count_is_refused_before_a_message_is_read(gbaes):
+    """One descriptor, passed off as 2^33."""
+    out = refused("lib.aes_ecb_batch_noalloc(msgs, 1 << 33, ctxs, 1, big, 16, big, 16, None)")
+    assert out.startswith("-1 ") and "too many messages" in out, out
 
 
 # ------------------------------------------------------------------------- GPU
