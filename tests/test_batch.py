@@ -114,6 +114,12 @@ def test_message_count_is_refused_before_a_message_is_read(gbaes):
     assert out.startswith("-1 ") and "too many messages" in out, out
 
 
+def test_bad_message_is_refused_without_memory_for_all_of_them(gbaes):
+    """The first of 2^32 - 16 messages names a key that is not there; 2 GiB are left to the process."""
+    out = refused("lib.aes_batch_tiles(msgs, 0xFFFFFFF0, ctxs, 1, 32, None, 0)", key=7, limit=2 << 30)
+    assert out.startswith("-1 ") and "message 0: key_index" in out, out
+
+
 # ------------------------------------------------------------------------- GPU
 
 torch = pytest.importorskip("torch")
