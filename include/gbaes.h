@@ -469,9 +469,13 @@ void aes_router_destroy(aes_router* router);
  * AES_KERNEL_TABLE at start).  Returns the previous variant or AES_ERR_ARG. */
 int aes_set_kernel(int which);
 
-/* Default launch shape of the table kernel for one (key size, direction):
- * threads per CTA (multiple of 32, 64..1024) and blocks per thread (1/2/4).
- * The autotuner calls this with the shape it measured fastest. */
+/* Sets the table kernel's launch shape for one key size and direction:
+ * threads per CTA (multiple of 32, 64..1024) and blocks per thread (1/2/4).  It
+ * holds for calls of every size, the ECB calls, CTR (encryption's shape; its
+ * long inputs have a kernel of their own), CBC decryption and the staged
+ * pipeline.  Until it is set, and again after 0, 0, the library chooses the
+ * shape by the size of each call.  The autotuner calls this with the shape it
+ * measured fastest. */
 int aes_set_tuning(int bits, int decrypt, int threads, int blocks_per_thread);
 
 /* Reads (and with clear != 0 resets) the library's device status word on the

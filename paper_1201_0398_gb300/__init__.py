@@ -313,6 +313,7 @@ def set_kernel(which: int) -> int:
 
 
 def set_tuning(bits: int, decrypt: bool, threads: int, blocks_per_thread: int) -> None:
+    """The table kernel's launch shape for one key size and direction, at every size; 0, 0: by size again."""
     _check(load().aes_set_tuning(int(bits), int(bool(decrypt)), int(threads), int(blocks_per_thread)))
 
 

@@ -433,8 +433,11 @@ int aes_set_tuning(int bits, int decrypt, int threads, int blocks_per_thread) {
     int bi = bits_index(bits);
     if (bi < 0) return fail(AES_ERR_KEYSIZE, "key size %d bits is not 128, 192 or 256", bits);
     if (decrypt != 0 && decrypt != 1) return fail(AES_ERR_ARG, "decrypt must be 0 or 1");
-    if (!valid_threads(threads)) return fail(AES_ERR_ARG, "threads %d: need a multiple of 32 in [64, 1024]", threads);
-    if (!valid_bpt(blocks_per_thread)) return fail(AES_ERR_ARG, "blocks_per_thread %d: need 1, 2 or 4", blocks_per_thread);
+    if (threads || blocks_per_thread) {  // (both 0: by size again)
+        if (!valid_threads(threads)) return fail(AES_ERR_ARG, "threads %d: need a multiple of 32 in [64, 1024]", threads);
+        if (!valid_bpt(blocks_per_thread))
+            return fail(AES_ERR_ARG, "blocks_per_thread %d: need 1, 2 or 4", blocks_per_thread);
+    }
     std::lock_guard<std::mutex> lk(g_tuning_mu);
     g_tuning[bi][decrypt] = Tuning{threads, blocks_per_thread};
     return AES_OK;

@@ -98,6 +98,9 @@ def test_kernel_and_tuning_argument_checks(gbaes):
     assert lib.aes_set_tuning(128, 0, 1000, 2) == -1
     assert lib.aes_set_tuning(128, 0, 1024, 3) == -1
     assert lib.aes_set_tuning(128, 0, 1024, 2) == 0
+    assert lib.aes_set_tuning(128, 0, 0, 2) == -1
+    assert lib.aes_set_tuning(128, 0, 1024, 0) == -1
+    assert lib.aes_set_tuning(128, 0, 0, 0) == 0  # the shape by size, as at the start
 
 
 def test_argument_checks_before_any_cuda_call(gbaes):
