@@ -432,7 +432,7 @@ GBAES_HD inline void add_key_half(uint32_t (&s)[64], const Keys& keys, int r) {
 
 // MixColumns on the half's two columns (after ShiftRows and SubBytes), each as a
 // generated program of two- and three-input XORs (sbox_lut3.h).  The round key
-// was added before it, transformed (see make_key_planes).
+// was added before it, transformed (see key_word).
 GBAES_HD inline void mix_half(uint32_t (&s)[64]) {
     mix_column_lut3(&s[0], Lop3{});
     mix_column_lut3(&s[32], Lop3{});
@@ -462,7 +462,7 @@ GBAES_HD inline void sub_bytes_key_half(uint32_t (&s)[64], const Keys& keys, int
     }
 }
 
-// Encryption of a half state, with the key planes of make_key_planes: step 0
+// Encryption of a half state, with the key planes of key_word: step 0
 // before the first round, step r (the affine constant plus InvMixColumns of
 // round key r, so that MixColumns turns it into round key r) on the S-box
 // output of round r.  ShiftRows runs before SubBytes: the two commute, one
@@ -487,7 +487,7 @@ GBAES_HD inline void encrypt_half(uint32_t (&s)[64], const Keys& keys, const Oth
 //   s' = InvMixColumns(A^-1 F(A^-1 InvShiftRows(s)) ^ k)
 // becomes, on t,
 //   t' = A^-1 InvMixColumns A^-1 (F(InvShiftRows(t)) ^ A k):
-// the encryption's S-box network with the key planes A k (make_key_planes),
+// the encryption's S-box network with the key planes A k (key_word),
 // then one linear map per column.  The last round has no InvMixColumns: the
 // output is A^-1 (F(InvShiftRows(t)) ^ A k).  The affine constant rides in the
 // key planes as before.
@@ -555,20 +555,17 @@ GBAES_HD inline uint32_t key_word(const uint32_t* rk, int nr, bool decrypt, int 
     return w;
 }
 
-// The same as planes (0 or all ones), plane p = 8*(state byte) + bit.
-GBAES_HD inline void make_key_planes(const uint32_t* rk, int nr, bool decrypt, uint32_t (*planes)[128]) {
+// The key words of every step, word c of step r at out[4 * r + c].
+GBAES_HD inline void make_key_words(const uint32_t* rk, int nr, bool decrypt, uint32_t* out) {
     for (int r = 0; r <= nr; ++r)
-        for (int c = 0; c < 4; ++c) {
-            const uint32_t w = key_word(rk, nr, decrypt, r, c);
-            for (int p = 0; p < 32; ++p) planes[r][32 * c + p] = ((w >> p) & 1u) ? 0xffffffffu : 0u;
-        }
+        for (int c = 0; c < 4; ++c) out[4 * r + c] = key_word(rk, nr, decrypt, r, c);
 }
 
-// Lays make_key_planes' output out for HalfKeys: step r, half h, local plane q
-// at out[kKeyStepWords*r + kKeyHalfWords*h + q] (q = p - 64h).
-GBAES_HD inline void split_key_planes(const uint32_t (*planes)[128], int nr, uint32_t* out) {
-    for (int r = 0; r <= nr; ++r)
-        for (int p = 0; p < 128; ++p) out[kKeyStepWords * r + kKeyHalfWords * (p / 64) + p % 64] = planes[r][p];
+// Plane i of all (plane i % 128 of step i / 128) from the key words, 0 or all ones, at its
+// place in the layout of HalfKeys: step r, half h, local plane q at
+// out[kKeyStepWords * r + kKeyHalfWords * h + q].
+GBAES_HD inline void put_key_plane(const uint32_t* words, int i, uint32_t* out) {
+    out[kKeyStepWords * (i >> 7) + kKeyHalfWords * ((i >> 6) & 1) + (i & 63)] = 0u - ((words[i >> 5] >> (i & 31)) & 1u);
 }
 
 }  // namespace bs

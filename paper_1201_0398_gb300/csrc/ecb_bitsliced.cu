@@ -46,9 +46,7 @@ __global__ void __launch_bounds__(kBsThreads, DEC ? kBsCtasPerSmDec : kBsCtasPer
     // Key planes from the key words, in the layout of HalfKeys.  (As an 8 KB launch
     // parameter built on the host, a plane at a time, they made a call of 4 KiB - 4 MiB take
     // 36 us (AES-256 48); now 12-14 (16-17).)
-    for (int i = threadIdx.x; i < (NR + 1) * 128; i += blockDim.x)
-        keys_s[bs::kKeyStepWords * (i >> 7) + bs::kKeyHalfWords * ((i >> 6) & 1) + (i & 63)] =
-            0u - ((a.keys[i >> 5] >> (i & 31)) & 1u);
+    for (int i = threadIdx.x; i < (NR + 1) * 128; i += blockDim.x) bs::put_key_plane(a.keys, i, keys_s);
     __syncthreads();
     pdl_wait();
     pdl_trigger();
@@ -111,8 +109,7 @@ int launch_bitsliced(const EcbArgs& e, const uint32_t* enc_rk, int nr, Mode mode
     a.in = e.in;
     a.out = e.out;
     a.nblocks = e.nblocks;
-    for (int r = 0; r <= nr; ++r)
-        for (int c = 0; c < 4; ++c) a.keys[4 * r + c] = bs::key_word(enc_rk, nr, dec, r, c);
+    bs::make_key_words(enc_rk, nr, dec, a.keys);
     DeviceInfo info;
     int rc = current_device_info(&info);
     if (rc) return rc;

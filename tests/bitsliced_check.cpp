@@ -70,10 +70,10 @@ int main() {
     if (fread(rk, 4, 4 * (nr + 1), stdin) != (size_t)(4 * (nr + 1))) return 1;
     uint32_t blocks[32][4];
     if (fread(blocks, 16, 32, stdin) != 32) return 1;
-    static uint32_t planes[15][128];
+    uint32_t words[60];
     static uint32_t split[15 * gbaes::bs::kKeyStepWords];
-    gbaes::bs::make_key_planes(rk, nr, dec != 0, planes);
-    gbaes::bs::split_key_planes(planes, nr, split);
+    gbaes::bs::make_key_words(rk, nr, dec != 0, words);
+    for (int i = 0; i < (nr + 1) * 128; ++i) gbaes::bs::put_key_plane(words, i, split);
     static uint32_t s[2][64];
     for (int h = 0; h < 2; ++h) {  // half h: words 2h, 2h+1 of every block, as the kernel loads them
         for (int k = 0; k < 32; ++k) {
