@@ -440,7 +440,7 @@ def run_ours(args):
     dom_name, dom = max(op_stats.items(), key=lambda kv: kv[1]["ms"])
     bits_dom = int(dom_name[3:6])
     dec_dom = dom_name.endswith("dec")
-    bpt_dom = tuned.get(dom_name, {}).get("blocks_per_thread", 2)
+    bpt_dom = tuned.get(dom_name, {}).get("blocks_per_thread", 0) or (1 if size // 16 <= 2 * sms * 512 else 2)
     ktpl = f"table_kernel<{NR[bits_dom]},{1 if dec_dom else 0},{bpt_dom}>"
     traffic = dram_traffic(f"table_kernel<{NR[bits_dom]},{1 if dec_dom else 0}>") if kernel == g.KERNEL_TABLE else None
     clock_frac = None

@@ -312,9 +312,18 @@ def set_kernel(which: int) -> int:
     return _check(load().aes_set_kernel(int(which)))
 
 
+_tuning = {}
+
+
 def set_tuning(bits: int, decrypt: bool, threads: int, blocks_per_thread: int) -> None:
     """The table kernel's launch shape for one key size and direction, at every size; 0, 0: by size again."""
     _check(load().aes_set_tuning(int(bits), int(bool(decrypt)), int(threads), int(blocks_per_thread)))
+    _tuning[int(bits), bool(decrypt)] = int(threads), int(blocks_per_thread)
+
+
+def tuning(bits: int, decrypt: bool) -> tuple:
+    """The shape that set_tuning was last called with; (0, 0), by size, at the start."""
+    return _tuning.get((int(bits), bool(decrypt)), (0, 0))
 
 
 def device_status(clear: bool = False) -> int:

@@ -1,7 +1,9 @@
 """Autotuner for the table kernel's launch shape.
 
 Times candidate (threads per CTA, blocks per thread) pairs with CUDA events on
-the launching stream and keeps the fastest.  Results are cached in a JSON file
+the launching stream and keeps the fastest; (0, 0) is the library's own choice,
+which depends on the size of each call, where another candidate holds for every
+size once it is set.  Results are cached in a JSON file
 keyed by (GPU name, key size, direction, size bucket) so a process pays the
 search once per GPU model.  The tuner only chooses among shapes the kernels
 were compiled for; it never changes what is computed (every shape is checked
@@ -15,10 +17,13 @@ import threading
 
 import numpy as np
 
-from . import KERNEL_TABLE, BatchPlan, Key, ecb_ex, load, set_tuning
+from . import KERNEL_TABLE, BatchPlan, Key, ecb_ex, load, set_tuning, tuning
 
-ECB_CANDIDATES = [(1024, 1), (1024, 2), (1024, 4), (768, 2), (768, 4), (512, 2), (512, 4)]
+ECB_CANDIDATES = [(0, 0), (1024, 1), (1024, 2), (1024, 4), (768, 2), (768, 4), (512, 2), (512, 4)]
 BATCH_CANDIDATES = [(1024, 2), (1024, 4), (1024, 1), (768, 2), (512, 4), (512, 8)]
+# Kept instead of the shape by size: a shape faster than it by more than this.  The shape by size
+# is one of the others at any one size (512 x 2 at 256 MiB), and two timings of one shape differ by up to 0.5%.
+ECB_MARGIN = 0.01
 _lock = threading.Lock()
 
 
@@ -70,7 +75,8 @@ def _time(fn, reps: int, stream) -> float:
 def tune_ecb(bits: int, decrypt: bool, nbytes: int = 256 << 20, reps: int = 10, force: bool = False,
              apply: bool = True) -> dict:
     """Best (threads, blocks_per_thread) of the table kernel for one key size and
-    direction on a buffer of nbytes; installs it as the default launch shape."""
+    direction on a buffer of nbytes, (0, 0) being the shape by size; installs it
+    as the default launch shape."""
     import torch
 
     load()
@@ -85,11 +91,18 @@ def tune_ecb(bits: int, decrypt: bool, nbytes: int = 256 << 20, reps: int = 10, 
         y = torch.empty_like(x)
         stream = torch.cuda.current_stream()
         times = {}
-        for threads, bpt in ECB_CANDIDATES:
-            ms = _time(lambda: ecb_ex(k, x, y, decrypt=decrypt, kernel=KERNEL_TABLE, threads=threads,
-                                      blocks_per_thread=bpt, stream=stream), reps, stream)
-            times[f"{threads}x{bpt}"] = ms
+        before = tuning(bits, decrypt)
+        set_tuning(bits, decrypt, 0, 0)  # what a call with 0, 0 runs
+        try:
+            for threads, bpt in ECB_CANDIDATES:
+                ms = _time(lambda: ecb_ex(k, x, y, decrypt=decrypt, kernel=KERNEL_TABLE, threads=threads,
+                                          blocks_per_thread=bpt, stream=stream), reps, stream)
+                times[f"{threads}x{bpt}"] = ms
+        finally:
+            set_tuning(bits, decrypt, *before)
         best = min(times, key=times.get)
+        if times["0x0"] <= times[best] * (1 + ECB_MARGIN):
+            best = "0x0"
         threads, bpt = (int(v) for v in best.split("x"))
         hit = {"threads": threads, "blocks_per_thread": bpt, "ms": times[best], "nbytes": nbytes,
                "gbs": nbytes / (times[best] / 1e3) / 1e9, "candidates_ms": times}
