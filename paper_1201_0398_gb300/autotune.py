@@ -4,13 +4,14 @@ Times candidate (threads per CTA, blocks per thread) pairs with CUDA events on
 the launching stream and keeps the fastest; (0, 0) is the library's own choice,
 which depends on the size of each call, where another candidate holds for every
 size once it is set.  Results are cached in a JSON file
-keyed by (GPU name, key size, direction, size bucket) so a process pays the
-search once per GPU model.  The tuner only chooses among shapes the kernels
+keyed by (GPU name, kernel sources, key size, direction, size bucket) so a
+process pays the search once per GPU model and version of the kernel.  The tuner only chooses among shapes the kernels
 were compiled for; it never changes what is computed (every shape is checked
 bit-exact by the tests).
 """
 from __future__ import annotations
 
+import hashlib
 import json
 import os
 import threading
@@ -53,6 +54,17 @@ def _save_cache(c: dict) -> None:
     os.replace(tmp, p)
 
 
+def _kernel_id() -> str:
+    """Hash of the table kernel's sources: shapes measured with another kernel say nothing about this one."""
+    from . import _build
+
+    h = hashlib.sha256()
+    for name in ("ecb_table.cu", "block_io.cuh", "aes_rounds.cuh", "launch.cuh"):
+        with open(os.path.join(_build.CSRC, name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
+
+
 def size_bucket(nbytes: int) -> int:
     """log4 bucket of a buffer size (4 KiB -> 6, 1 MiB -> 10, 1 GiB -> 15)."""
     return int(np.floor(np.log(max(nbytes, 16)) / np.log(4)))
@@ -81,7 +93,7 @@ def tune_ecb(bits: int, decrypt: bool, nbytes: int = 256 << 20, reps: int = 10, 
 
     load()
     name = torch.cuda.get_device_name()
-    key = f"ecb|{name}|{bits}|{int(bool(decrypt))}|{size_bucket(nbytes)}"
+    key = f"ecb|{name}|{_kernel_id()}|{bits}|{int(bool(decrypt))}|{size_bucket(nbytes)}"
     with _lock:
         cache = _load_cache()
         hit = cache.get(key)

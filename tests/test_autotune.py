@@ -40,3 +40,19 @@ def test_the_shape_by_size_stays_unless_another_is_faster(gbaes, tuner):
     tuner.times[512, 4] = 0.8
     hit = tuner.tune_ecb(128, False, nbytes=1 << 16, force=True, apply=False)
     assert (hit["threads"], hit["blocks_per_thread"]) == (512, 4) and gbaes.tuning(128, False) == (1024, 2)
+
+
+@pytest.mark.gpu
+def test_shapes_of_another_kernel_are_not_used(gbaes, tuner):
+    """Entries of a cache file written by other kernel sources, or before it named them."""
+    tuner.times[1024, 2] = 0.9
+    first = tuner.tune_ecb(128, False, nbytes=1 << 16)
+    assert tuner.tune_ecb(128, False, nbytes=1 << 16) == first  # (from the file)
+    with open(tuner.cache_path()) as f:
+        (key, hit), = json.load(f).items()
+    name, kernel, rest = key.split("|", 1)[1].split("|", 2)
+    for other in (f"ecb|{name}|{rest}", f"ecb|{name}|{'0' * len(kernel)}|{rest}"):
+        with open(tuner.cache_path(), "w") as f:
+            json.dump({other: dict(hit, threads=768, blocks_per_thread=4)}, f)
+        got = tuner.tune_ecb(128, False, nbytes=1 << 16)
+        assert (got["threads"], got["blocks_per_thread"]) == gbaes.tuning(128, False) == (1024, 2)
