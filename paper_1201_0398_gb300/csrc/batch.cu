@@ -336,7 +336,6 @@ int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ct
     uint32_t count[kGroups] = {};
     uint64_t blocks[kGroups] = {};
     std::vector<uint8_t> group;  // of each message; kGroups: no blocks.  Grows with the messages found valid.
-    group.reserve(std::min<size_t>(nmsg, 1 << 16));
     for (size_t i = 0; i < nmsg; ++i) {
         const aes_msg_desc& m = d[i];
         if (m.key_index >= nctx) return fail(AES_ERR_ARG, "message %zu: key_index %u >= %zu", i, m.key_index, nctx);
@@ -346,14 +345,13 @@ int build_host_plan(const aes_msg_desc* d, size_t nmsg, const aes_ctx* const* ct
         const uint64_t bytes = m.nblocks * 16;
         if (m.in_off > UINT64_MAX - bytes || m.out_off > UINT64_MAX - bytes)
             return fail(AES_ERR_ARG, "message %zu: offset + length overflows", i);
-        if (m.nblocks == 0) {
-            group.push_back(kGroups);
-            continue;
-        }
+        if (i == group.size()) group.resize(std::min(nmsg, std::max<size_t>(2 * i, 1 << 20)));
+        group[i] = kGroups;
+        if (m.nblocks == 0) continue;
         P->in_extent = std::max<uint64_t>(P->in_extent, m.in_off + bytes);
         P->out_extent = std::max<uint64_t>(P->out_extent, m.out_off + bytes);
         const int g = group_of(ctxs[m.key_index]->nr, (int)m.decrypt);
-        group.push_back((uint8_t)g);
+        group[i] = (uint8_t)g;
         ++count[g];
         blocks[g] += m.nblocks;
     }
