@@ -578,32 +578,49 @@ int launch_batch_kernel(const HostPlan& H, BatchArgs a, int threads, int bpt, cu
     return AES_OK;
 }
 
-// Tile size and launch shape of a call that plans for one launch (kept plans
-// take theirs from the caller).
+// Largest tile of a call that plans for one launch, in blocks.
 constexpr uint32_t kOneShotTileMax = 2048;
 
-struct OneShot {
-    uint32_t tile_blocks;
-    int threads, bpt;
-};
-
-// From this many blocks on a launch whose shape the caller left open runs 512
-// threads x 8 blocks instead of 1024 x 2: a warp reads each round's key for 8 states
-// instead of 2 (4 cycles of the L1 data stage per read, beside 16 per state), which
-// counts once unit starts and tails do not.  1024 x 2 against 512 x 8, messages up to
-// 4 MiB: 42.5 / 44.7 us at 24 MB, 124 / 124 at 89 MB, 213 / 210 at 149 MB, 315 / 305 at
-// 231 MB, 397 / 384 at 294 MB, 1,218 / 1,175 at 918 MB, 4,395 / 4,235 at 3.4 GB; shorter
-// messages: 205 / 242 at 146 MB (up to 128 KiB), 10.3 / 19.0 at 4.7 MB (up to 16 KiB).
-constexpr uint64_t kWideBlocks = 3ull << 22;
-
-// Above 2^23 blocks tiles of 512 would only lengthen the upload.
-static OneShot one_shot_shape(const aes_msg_desc* d, size_t nmsg) {
+// Tiles of 512 blocks, which above 2^23 blocks would only lengthen the upload.
+static uint32_t one_shot_tile(const aes_msg_desc* d, size_t nmsg) {
     uint64_t total = 0;
     if (nmsg > kMaxMessages) nmsg = 0;  // (build_host_plan refuses the count before it reads a message)
     for (size_t i = 0; d && i < nmsg; ++i) total += std::min<uint64_t>(d[i].nblocks, 1ull << 32);
-    if (total <= 1u << 23) return OneShot{512, 1024, 2};
-    if (total < kWideBlocks) return OneShot{kOneShotTileMax, 1024, 2};
-    return OneShot{kOneShotTileMax, 512, 8};
+    return total <= 1u << 23 ? 512 : kOneShotTileMax;
+}
+
+// A launch whose shape the caller left open runs 1024 threads x 2 blocks, or 512 x 8:
+// there a warp reads each round's key for 8 states instead of 2 (4 cycles of the L1
+// data stage per read, beside 16 per state), which counts from kWideBlocks on, once
+// unit starts and tails do not; but a message that starts inside a pass makes all 256
+// blocks of it, not 64, read keys for each state.  512 x 8
+// over 1024 x 2, kept plans of 190 MB to 1.8 GB, by the share of such passes: none 0.961-0.988,
+// 0.8% 0.964-1.000, 2.5% 0.971-0.996, 4.5% 0.979-1.000 (messages up to 512 KiB), 8% 0.991-1.026
+// (up to 256 KiB), 14% 1.017-1.062, 23% 1.089-1.150, 60% 1.25-1.29 (up to 16 KiB).  By size,
+// messages up to 4 MiB: 42.5 us with 1024 x 2 and 44.7 with 512 x 8 at 24 MB, 124 / 124 at
+// 89 MB, 213 / 210 at 149 MB, 315 / 305 at 231 MB, 1,218 / 1,175 at 918 MB, 4,395 / 4,235 at 3.4 GB.
+constexpr uint64_t kWideBlocks = 3ull << 22;
+constexpr uint64_t kWidePass = 256;     // blocks of a warp's pass with 8 blocks per thread
+constexpr uint64_t kWideCrossed = 20;  // at most one pass in this many crossed
+
+struct Shape {
+    int threads, bpt;
+};
+
+static Shape open_shape(const HostPlan& H) {
+    const Shape narrow{1024, 2}, wide{512, 8};
+    if (H.total_blocks < kWideBlocks) return narrow;
+    uint64_t left = H.total_blocks / kWidePass / kWideCrossed;
+    for (const GroupDev& G : H.groups) {
+        uint64_t last = UINT64_MAX;  // the pass that was counted last
+        for (uint32_t m = G.msg_start; m < G.msg_end; ++m) {
+            const uint64_t start = H.msgs[m].blk_start;
+            if (start % kWidePass == 0 || start / kWidePass == last) continue;
+            if (left-- == 0) return narrow;
+            last = start / kWidePass;
+        }
+    }
+    return wide;
 }
 
 }  // namespace gbaes
@@ -643,9 +660,10 @@ aes_batch_plan* aes_batch_plan_create(const aes_msg_desc* msgs, size_t nmsg, con
         delete P;
         return nullptr;
     }
-    if (open && P->host.total_blocks >= kWideBlocks) {  // (the tiles stay 1024 x 2's)
-        P->threads = 512;
-        P->bpt = 8;
+    if (open) {  // (the tiles stay 1024 x 2's)
+        const Shape shape = open_shape(P->host);
+        P->threads = shape.threads;
+        P->bpt = shape.bpt;
     }
     if (cudaGetDevice(&P->device) != cudaSuccess) {
         fail(AES_ERR_CUDA, "no CUDA device");
@@ -780,8 +798,7 @@ int aes_ecb_batch(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* c
                     "aes_ecb_batch uploads from host memory freed on return and cannot be captured; "
                     "use aes_batch_plan_launch_graph");
     HostPlan H;
-    const OneShot shape = one_shot_shape(msgs, nmsg);
-    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, &H);
+    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, one_shot_tile(msgs, nmsg), &H);
     if (rc) return rc;
     if (H.ntiles == 0) return AES_OK;
     rc = check_bases(H, in_base, in_bytes, out_base, out_bytes);
@@ -803,6 +820,7 @@ int aes_ecb_batch(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* c
     a.in = (const uint4*)in_base;
     a.out = (uint4*)out_base;
     tables.fill_args(H, buf, &a);
+    const Shape shape = open_shape(H);
     rc = launch_batch_kernel(H, a, shape.threads, shape.bpt, s);
     cudaFreeAsync(buf, s);
     return rc;
@@ -873,13 +891,11 @@ extern "C" {
 int aes_ecb_batch_noalloc(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* const* ctxs, size_t nctx,
                           const void* in_base, size_t in_bytes, void* out_base, size_t out_bytes, void* stream) {
     HostPlan H;
-    OneShot shape = one_shot_shape(msgs, nmsg);
-    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, &H);
+    int rc = build_host_plan(msgs, nmsg, ctxs, nctx, one_shot_tile(msgs, nmsg), &H);
     if (rc) return rc;
-    if (Tables(H, nctx).bytes > kNoAllocScratchBytes && shape.tile_blocks != kOneShotTileMax) {
-        shape.tile_blocks = kOneShotTileMax;  // the smallest tables
+    if (Tables(H, nctx).bytes > kNoAllocScratchBytes && H.tile_blocks != kOneShotTileMax) {
         H = HostPlan();
-        rc = build_host_plan(msgs, nmsg, ctxs, nctx, shape.tile_blocks, &H);
+        rc = build_host_plan(msgs, nmsg, ctxs, nctx, kOneShotTileMax, &H);  // the smallest tables
         if (rc) return rc;
     }
     if (H.ntiles == 0) return AES_OK;
@@ -905,6 +921,7 @@ int aes_ecb_batch_noalloc(const aes_msg_desc* msgs, size_t nmsg, const aes_ctx* 
     a.in = (const uint4*)in_base;
     a.out = (uint4*)out_base;
     tables.fill_args(H, buf, &a);
+    const Shape shape = open_shape(H);
     return launch_batch_kernel(H, a, shape.threads, shape.bpt, s);
 }
 

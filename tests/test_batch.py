@@ -4,6 +4,7 @@ Every message of a batch must come out exactly as the CPU oracle computes it
 and exactly as the single-message kernel computes it alone (AES output is
 unique, so "the same alone and in the mix" is bit equality)."""
 import os
+import re
 import subprocess
 import sys
 
@@ -236,6 +237,47 @@ def test_batch_whole_tiles_at_a_time(gbaes, threads, bpt, longest, total):
     for graph in (False, True, False):
         y.zero_()
         plan.launch(x, y, graph=graph)
+        assert torch.equal(y, want)
+
+
+def batch_kernels(call):
+    """Blocks per thread of the batched kernels that call() launches (more than once, should the profiler, as it
+    starts, miss the first launches)."""
+    for _ in range(3):
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            call()
+            torch.cuda.synchronize()
+        got = [int(m[1]) for e in prof.events() for m in [re.search(r"batch_kernel<(\d)", e.name)] if m]
+        if got:
+            break
+    return got
+
+
+# Where the launch shape is left open: one-shot calls plan in larger tiles above 2^23 blocks, and from 3 * 2^22 on
+# batches in which few passes of 256 blocks are crossed by a message's start run 8 blocks per thread.
+@pytest.mark.gpu
+@pytest.mark.parametrize("lengths", ("short", "long"))
+@pytest.mark.parametrize("total", (1 << 23, (1 << 23) + 1, (3 << 22) - 1, 3 << 22))
+def test_batch_of_open_shape(gbaes, total, lengths):
+    rng = np.random.default_rng(total)
+    nblocks = rng.integers(1, 601, total // 300) if lengths == "short" else rng.integers(3000, 120_001, total // 30_000)
+    nblocks = nblocks[:np.searchsorted(np.cumsum(nblocks), total)]
+    nblocks = np.append(nblocks, total - nblocks.sum())
+    n = len(nblocks)
+    ks = [gbaes.Key(rng.integers(0, 256, b // 8, dtype=np.uint8).tobytes()) for b in (128, 192, 256) * 20]
+    key_index, decrypt = rng.integers(0, len(ks), n), rng.integers(0, 2, n)
+    off = (np.cumsum(nblocks) - nblocks) * 16
+    x = torch.randint(0, 256, (16 * total,), dtype=torch.uint8, device="cuda")
+    want, y = torch.zeros_like(x), torch.zeros_like(x)
+    for i in range(n):
+        a, b = int(off[i]), int(off[i] + 16 * nblocks[i])
+        (gbaes.decrypt_ecb if decrypt[i] else gbaes.encrypt_ecb)(ks[key_index[i]], x[a:b], want[a:b])
+    d = gbaes.make_descs(off, off, nblocks, key_index, decrypt)
+    plan = gbaes.BatchPlan(d, ks)
+    bpt = 8 if total >= 3 << 22 and lengths == "long" else 2
+    for call in (lambda: plan.launch(x, y), lambda: plan.launch(x, y, graph=True), lambda: gbaes.ecb_batch(d, ks, x, y)):
+        y.zero_()
+        assert batch_kernels(call) == [bpt]
         assert torch.equal(y, want)
 
 
