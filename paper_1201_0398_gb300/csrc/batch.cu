@@ -44,6 +44,15 @@ __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefe
 
 constexpr uint32_t kNoBoundary = 0x7fffffffu;
 
+// Blocks per thread of the passes that messages start in.  A body of 8 states there, beside
+// the one of the passes that lie in one message, is too much for the instruction cache:
+// 512 x 8, 3,000 messages of 8,208 bytes (25 MB) 72.3 us with 8, 3.5 cycles of instruction fetch
+// per instruction issued (0.5 with the shorter rounds of four tables, 59.6 us), 56.6 with 4;
+// 10,000 messages up to 16 KiB (23 MB) 69.8 -> 54.0, up to 64 KiB (77 MB) 139.6 -> 127.2, up to
+// 128 KiB (141 MB) 240 -> 221, up to 4 MiB (3.2 GB) 4,102 -> 4,104.  With 2: 51.5, 49.1, 126.9, 216
+// and 4,105, but 5-20% more than 4 in batches of up to 5 MB.
+constexpr int kMixedBpt = 4;
+
 // Starts of the messages after `base`, relative to tb0: lane l gets message
 // base + 1 + l's (kNoBoundary past the group's last message or far away; 0 for
 // any start at or before tb0).  One coalesced load tells a warp where 32
@@ -192,12 +201,13 @@ __device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupD
         }
     }
     constexpr uint32_t kPass = 32u * BPT;
+    constexpr int kMixed = BPT < kMixedBpt ? BPT : kMixedBpt;
     const bool crossing = __any_sync(0xffffffffu, starts != 0u && starts < n);
     if (!JOINED) {
         if (!crossing)
             single_message_unit<DEC, BPT>(a, G, m, tb0, n, lane, L, kslot);
         else
-            mixed_passes<DEC, BPT>(a, G, m, starts, tb0, 0, n, n, lane, L);
+            mixed_passes<DEC, kMixed>(a, G, m, starts, tb0, 0, n, n, lane, L);
         return;
     }
     // Whole passes up to the next message's start (or the end) run with one message's
@@ -216,7 +226,8 @@ __device__ __forceinline__ void batch_warp_unit(const BatchArgs& a, const GroupD
             m += next == it;
             len = 0;
         } else {
-            mixed_passes<DEC, BPT>(a, G, m, starts, tb0, it, it + 1, n, lane, L);
+            const uint32_t stop = BPT == kMixed ? it + 1 : it + kPass < n ? it + kPass : n;
+            mixed_passes<DEC, kMixed>(a, G, m, starts, tb0, it, stop, n, lane, L);
             it += kPass;
         }
     }
@@ -594,14 +605,14 @@ static uint32_t one_shot_tile(const aes_msg_desc* d, size_t nmsg) {
 // data stage per read, beside 16 per state), which counts from kWideBlocks on, once
 // unit starts and tails do not; but a message that starts inside a pass makes all 256
 // blocks of it, not 64, read keys for each state.  512 x 8
-// over 1024 x 2, kept plans of 190 MB to 1.8 GB, by the share of such passes: none 0.961-0.988,
-// 0.8% 0.964-1.000, 2.5% 0.971-0.996, 4.5% 0.979-1.000 (messages up to 512 KiB), 8% 0.991-1.026
-// (up to 256 KiB), 14% 1.017-1.062, 23% 1.089-1.150, 60% 1.25-1.29 (up to 16 KiB).  By size,
+// over 1024 x 2, kept plans of 190-910 MB, by the share of such passes: 0.8% 0.961-1.000,
+// 2.5% 0.970-0.990, 4.5% 0.977-1.000 (messages up to 512 KiB), 8% 0.984-1.011 (up to 256 KiB),
+// 14% 0.999-1.030, 23% 1.019-1.055, 60% 1.07-1.10 (up to 16 KiB).  By size,
 // messages up to 4 MiB: 42.5 us with 1024 x 2 and 44.7 with 512 x 8 at 24 MB, 124 / 124 at
 // 89 MB, 213 / 210 at 149 MB, 315 / 305 at 231 MB, 1,218 / 1,175 at 918 MB, 4,395 / 4,235 at 3.4 GB.
 constexpr uint64_t kWideBlocks = 3ull << 22;
 constexpr uint64_t kWidePass = 256;     // blocks of a warp's pass with 8 blocks per thread
-constexpr uint64_t kWideCrossed = 20;  // at most one pass in this many crossed
+constexpr uint64_t kWideCrossed = 12;  // at most one pass in this many crossed
 
 struct Shape {
     int threads, bpt;
