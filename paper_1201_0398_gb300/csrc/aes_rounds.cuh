@@ -84,28 +84,41 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint32_t v) {
 
 // Writes one direction's table at A (16-byte aligned); threads tid = 0..nt-1 take
 // part and the caller synchronises them.  Four threads share an entry's 128 bytes:
-// thread p writes two 16-byte pieces of entry p / 4, the pieces rotated so that the
-// 8 threads of a quarter-warp's store hit 8 different bank groups.  A thread loads
-// up to four entries before storing any.
-__device__ __forceinline__ void fill_table(uint32_t A, bool decrypt, uint32_t tid, uint32_t nt) {
+// piece p in 0..1023 is two of the eight 16-byte parts of entry p / 4, rotated so
+// that the 8 threads of a quarter-warp's store hit 8 different bank groups.  A thread
+// loads the entries of up to kFillChunk pieces (p0 and every nt after it) before
+// storing any.
+constexpr uint32_t kFillPieces = 1024, kFillChunk = 4;
+
+__device__ __forceinline__ void fill_load(bool decrypt, uint32_t p0, uint32_t nt, uint32_t (&v)[kFillChunk]) {
     const uint32_t* t0 = decrypt ? g_tab.td0 : g_tab.te0;
-    for (uint32_t p0 = tid; p0 < 1024u; p0 += 4u * nt) {
-        uint32_t v[4];
 #pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) {
-            const uint32_t p = p0 + u * nt;
-            v[u] = p < 1024u ? __ldg(t0 + (p >> 2)) : 0u;
-        }
+    for (uint32_t u = 0; u < kFillChunk; ++u) {
+        const uint32_t p = p0 + u * nt;
+        v[u] = 0u;
+        // (volatile: issued here, ahead of what stands between this and fill_store)
+        if (p < kFillPieces) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v[u]) : "l"(t0 + (p >> 2)));
+    }
+}
+
+__device__ __forceinline__ void fill_store(uint32_t A, uint32_t p0, uint32_t nt, const uint32_t (&v)[kFillChunk]) {
 #pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) {
-            const uint32_t p = p0 + u * nt;
-            if (p < 1024u) {
-                const uint32_t piece = 2u * (p & 3u) + ((p >> 2) & 1u);
-                const uint32_t base = A + (p >> 2) * 128u;
-                sts128(base + 16u * piece, v[u]);
-                sts128(base + 16u * (piece ^ 1u), v[u]);
-            }
+    for (uint32_t u = 0; u < kFillChunk; ++u) {
+        const uint32_t p = p0 + u * nt;
+        if (p < kFillPieces) {
+            const uint32_t part = 2u * (p & 3u) + ((p >> 2) & 1u);
+            const uint32_t base = A + (p >> 2) * 128u;
+            sts128(base + 16u * part, v[u]);
+            sts128(base + 16u * (part ^ 1u), v[u]);
         }
+    }
+}
+
+__device__ __forceinline__ void fill_table(uint32_t A, bool decrypt, uint32_t tid, uint32_t nt) {
+    for (uint32_t p = tid; p < kFillPieces; p += kFillChunk * nt) {
+        uint32_t v[kFillChunk];
+        fill_load(decrypt, p, nt, v);
+        fill_store(A, p, nt, v);
     }
 }
 

@@ -57,7 +57,14 @@ __global__ void __launch_bounds__(1024, 1) table_kernel(const EcbArgs a) {
     constexpr bool kAhead = BPT <= 2;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t A = smem_base(smem_raw);
-    fill_table(A, DECRYPT, threadIdx.x, blockDim.x);
+    // The table's last pieces stay in registers until the first blocks' loads are out,
+    // where those come first.
+    uint32_t piece[kFillChunk], p = threadIdx.x;
+    for (; p + kFillChunk * blockDim.x < kFillPieces; p += kFillChunk * blockDim.x) {
+        fill_load(DECRYPT, p, blockDim.x, piece);
+        fill_store(A, p, blockDim.x, piece);
+    }
+    fill_load(DECRYPT, p, blockDim.x, piece);
     const uint32_t L = A + 4u * (threadIdx.x & 31u);
     const uint32_t step = blockDim.x;
     const uint64_t stride = (uint64_t)step * BPT * gridDim.x;  // blocks of one pass of every CTA
@@ -68,10 +75,15 @@ __global__ void __launch_bounds__(1024, 1) table_kernel(const EcbArgs a) {
     if (end > n) end = n;
     uint32_t next[BPT][4];
     uint4 next_aux[BPT];  // CTR: data; CBC: previous ciphertext block
-    pdl_wait();
-    if (kAhead) {
-        const bool full = i < first;
-        load_blocks<MODE, BPT>(a, full ? i : rest, step, full ? first : end, next, next_aux);
+    const bool any = i < first;
+    if (a.loads_first) {
+        pdl_wait();
+        if (kAhead) load_blocks<MODE, BPT>(a, any ? i : rest, step, any ? first : end, next, next_aux);
+    }
+    fill_store(A, p, blockDim.x, piece);
+    if (!a.loads_first) {
+        pdl_wait();
+        if (kAhead) load_blocks<MODE, BPT>(a, any ? i : rest, step, any ? first : end, next, next_aux);
     }
     __syncthreads();
     pdl_trigger();  // (after the barrier: 0.2 us less per call than at the kernel's start)
@@ -230,12 +242,13 @@ __global__ void __launch_bounds__(256) table_compact_kernel(const EcbArgs a) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t T = smem_base(tab);
-    fill_compact(T, DECRYPT);
-    pdl_wait();
-    pdl_trigger();
     uint32_t s[4];
     uint4 aux;
+    if (!a.loads_first) fill_compact(T, DECRYPT);
+    pdl_wait();
+    pdl_trigger();
     load_block<MODE>(a, i, i < n, s, aux);
+    if (a.loads_first) fill_compact(T, DECRYPT);
     __syncthreads();
     while (i < n) {
         cipher_compact<NR, DECRYPT>(s, ParamKeys{a.rk}, T);
@@ -294,7 +307,7 @@ constexpr int kMinThreads = 128;
 
 uint64_t compact_limit_blocks(int sms) { return (uint64_t)sms * kCompactBlocksPerSm; }
 
-int launch_table(const EcbArgs& a, int nr, Mode mode, int threads, int bpt, int variant, cudaStream_t stream) {
+int launch_table(EcbArgs a, int nr, Mode mode, int threads, int bpt, int variant, cudaStream_t stream) {
     DeviceInfo info;
     int rc = current_device_info(&info);
     if (rc) return rc;
@@ -340,7 +353,9 @@ int launch_table(const EcbArgs& a, int nr, Mode mode, int threads, int bpt, int 
             if (rc) return rc;
         }
     }
-    const cudaError_t e = launch_overlapped(fn, grid, (unsigned)threads, (size_t)smem, stream, a);
+    const bool overlap = may_overlap(stream);
+    a.loads_first = !overlap;
+    const cudaError_t e = launch_overlapped(fn, grid, (unsigned)threads, (size_t)smem, stream, a, overlap);
     if (e != cudaSuccess) return fail(AES_ERR_CUDA, "table kernel launch: %s", cudaGetErrorString(e));
     return AES_OK;
 }

@@ -39,6 +39,7 @@ struct EcbArgs {
     uint64_t first;    // kCtr: counter index of in[0]
     uint32_t iv[4];    // kCbcDec: ciphertext block before in[0]
     int ctr_be;        // kCtr: 1 = big-endian 128-bit counter, 0 = little-endian words
+    int loads_first;   // set by launch_table: the first blocks are loaded before the tables are filled
 };
 
 struct DeviceInfo {
@@ -81,7 +82,7 @@ uint64_t compact_limit_blocks(int sms);
 // Launches the T-table kernel (ecb_table.cu).  variant: AES_KERNEL_TABLE (picks
 // by size), AES_KERNEL_TABLE_COMPACT or AES_KERNEL_TABLE_REPLICATED; threads
 // and bpt shape the replicated kernel only.
-int launch_table(const EcbArgs& a, int nr, Mode mode, int threads, int bpt, int variant, cudaStream_t stream);
+int launch_table(EcbArgs a, int nr, Mode mode, int threads, int bpt, int variant, cudaStream_t stream);
 
 // CTR on inputs of at least ctr_min_blocks blocks (ctr.cu); a.first is any 64-bit index.
 uint64_t ctr_min_blocks(int sms);

@@ -9,8 +9,10 @@
 // before it in the stream to have ended and its writes to be visible.  Measured on a
 // stream of such calls, before and after: 4 KiB 4.10 -> 2.6 us (host bound), 1 MiB 6.15 ->
 // 2.75, 9 MiB 15.8 -> 12.0, 64 MiB 79.9 -> 74.6.  Filling the tables before the wait
-// instead of after it is 0.7 us of that, and costs a call on its own nothing that
-// could be measured (the first block's load no longer overlaps the fill).
+// instead of after it is 0.7 us of that.  Where there is no predecessor to wait for,
+// the fill would only keep the first blocks' loads waiting (4 KiB in a captured graph
+// 2.32 us with the loads first, 2.46 with the fill first; up to 300 KiB 0.12-0.2 us):
+// the single-call kernels take their loads first in a plain launch (EcbArgs::loads_first).
 //
 // Every kernel launched here calls pdl_wait in every thread before it touches
 // global memory other than constants of the library, and pdl_trigger once.  A
@@ -29,11 +31,22 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // Lets the next kernel of the stream start (once every CTA has called this or ended).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// fn<<<grid, threads, smem, stream>>>(a), overlapping its predecessor.  A stream
-// being captured gets a plain launch, so that a captured graph has ordinary edges.
+// Whether the next kernel of the stream may overlap its predecessor: not while the
+// stream is being captured, so that a captured graph has ordinary edges.
+inline bool may_overlap(cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+        cudaGetLastError();  // (the legacy stream beside a capture: the launch reports it)
+        return false;
+    }
+    return cap == cudaStreamCaptureStatusNone;
+}
+
+// fn<<<grid, threads, smem, stream>>>(a), overlapping its predecessor or (overlap
+// false) a plain launch, in which pdl_wait returns at once.
 template <class Args>
 cudaError_t launch_overlapped(void (*fn)(Args), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
-                              const Args& a) {
+                              const Args& a, bool overlap) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
@@ -42,14 +55,17 @@ cudaError_t launch_overlapped(void (*fn)(Args), unsigned grid, unsigned threads,
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
-        cudaGetLastError();  // (the legacy stream beside a capture: the launch reports it)
-    } else if (cap == cudaStreamCaptureStatusNone) {
+    if (overlap) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
     }
     return cudaLaunchKernelEx(&cfg, fn, a);
+}
+
+template <class Args>
+cudaError_t launch_overlapped(void (*fn)(Args), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
+                              const Args& a) {
+    return launch_overlapped(fn, grid, threads, smem, stream, a, may_overlap(stream));
 }
 #endif
 

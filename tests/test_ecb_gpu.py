@@ -3,6 +3,7 @@
 AES is a permutation per key, so the result is unique and the tolerance is zero
 (Section 2.1's cipher; Eq. 1 is a re-arrangement of the same arithmetic).
 """
+import ctypes
 import json
 import os
 
@@ -541,4 +542,53 @@ def test_dependent_calls_on_buffers_off_by_a_block(gbaes, n):
     assert np.array_equal(host(x), want)
     for b in bufs:  # nothing before or after the blocks
         assert not host(b[:16]).any() and not host(b[16 * (n + 1):]).any()
+    assert gbaes.device_status() == 0
+
+
+@pytest.mark.parametrize("bits", BITS)
+@pytest.mark.parametrize("captured", (False, True))
+def test_short_calls_in_both_orders(gbaes, bits, captured):
+    """A plain launch (a captured call) loads its first blocks before it fills its
+    table, an overlapped one after: short calls of every mode, table variant and
+    number of fill steps per thread (CTAs of 64 to 1024 threads), at one block, at
+    whole and ragged shares of a CTA, and on both sides of the lines by size."""
+    rng = np.random.default_rng(2100 + bits)
+    key = rng.integers(0, 256, bits // 8, dtype=np.uint8).tobytes()
+    iv = rng.integers(0, 256, 16, dtype=np.uint8).tobytes()
+    k = gbaes.Key(key)
+    s = sms()
+    shapes = [(gbaes.KERNEL_TABLE, 0, 0), (gbaes.KERNEL_TABLE_COMPACT, 0, 0)]
+    shapes += [(gbaes.KERNEL_TABLE_REPLICATED, t, b) for t, b in ((64, 1), (96, 2), (128, 4), (256, 1), (512, 2), (1024, 4))]
+    sizes = (1, 33, 32 * s, 64 * s - 1, 64 * s + 1, 128 * s, 128 * s + 1, 256 * s + 31)
+    data = rng.integers(0, 256, 16 * max(sizes), dtype=np.uint8)
+    x = dev(data)
+    iv_c = (ctypes.c_uint8 * 16)(*iv)
+    lib = gbaes.load()
+    calls = [(oracle.ecb(key, bits, data, decrypt=d),
+              lambda n, y, s, d=d, v=v: lib.aes_ecb_ex(k.handle, int(d), x.data_ptr(), y.data_ptr(), n, *v, s))
+             for d in (False, True) for v in shapes]
+    calls += [(oracle.ctr(key, bits, iv, data),
+               lambda n, y, s: lib.aes_ctr_xcrypt(k.handle, iv_c, 0, 0, x.data_ptr(), y.data_ptr(), n, s)),
+              (oracle.cbc_decrypt(key, bits, iv, data),
+               lambda n, y, s: lib.aes_cbc_decrypt(k.handle, iv_c, x.data_ptr(), y.data_ptr(), n, s))]
+    stream = torch.cuda.Stream()
+    outs = [torch.zeros_like(x) for _ in calls]
+    torch.cuda.synchronize()
+    for n in sizes:
+        def go():
+            for (_, call), y in zip(calls, outs):
+                assert call(n, y, stream.cuda_stream) == 0
+
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream):
+                go()
+            g.replay()
+        else:
+            go()
+        torch.cuda.synchronize()
+        for i, ((want, _), y) in enumerate(zip(calls, outs)):
+            assert np.array_equal(host(y[:16 * n]), want[:16 * n]), (n, i)
+            assert not y[16 * n:].any(), (n, i)
+            y.zero_()
     assert gbaes.device_status() == 0
