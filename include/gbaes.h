@@ -55,11 +55,11 @@ extern "C" {
 
 /* Kernel variants for aes_ecb_ex / aes_set_kernel. */
 #define AES_KERNEL_TABLE 0     /* Eq. 1 T-table kernel, tables in shared memory: the replicated
-                                  tables, or the compact ones for calls too small to fill the GPU */
+                                  one at every size */
 #define AES_KERNEL_BITSLICED 1 /* Boolean-circuit S-box over bit planes of 32 blocks */
 #define AES_KERNEL_TABLE_COMPACT 2    /* T-table kernel with each table stored once (4-5 KiB of shared
                                          memory, cheap to fill; lookups may meet bank conflicts), any
-                                         size; its launch shape is its own (threads and
+                                         size, only where it is asked for; its launch shape is its own (threads and
                                          blocks_per_thread are ignored) */
 #define AES_KERNEL_TABLE_REPLICATED 3 /* T-table kernel with 32 lane copies of its table (bank-conflict
                                          free, 32 KiB to fill per CTA), any size */
@@ -105,7 +105,9 @@ int aes_decrypt_ecb(const aes_ctx* ctx, const void* in, void* out, size_t nblock
  * [64, 1024] (0 = default; checked, but the bitsliced kernel always runs
  * 128-thread CTAs, its shape fixed by its register budget).
  * blocks_per_thread: 1, 2 or 4 for the table kernel (0 = default; the
- * bitsliced kernel always holds 32 blocks per pair of lanes). */
+ * bitsliced kernel always holds 32 blocks per pair of lanes).  With
+ * AES_KERNEL_TABLE, calls of up to 128 blocks per SM run in a shape of their
+ * own whatever is given; AES_KERNEL_TABLE_REPLICATED takes the shape given. */
 int aes_ecb_ex(const aes_ctx* ctx, int decrypt, const void* in, void* out, size_t nblocks, int kernel,
                int threads, int blocks_per_thread, void* stream);
 

@@ -126,23 +126,17 @@ __global__ void __launch_bounds__(1024, 1) table_kernel(const EcbArgs a) {
 
 // ------------------------------------------------------------ compact tables
 //
-// Calls too small to fill the GPU are bound by latency, not by the lookup rate:
-// the 32x replicated table (32 KiB per CTA) takes longer to write than the few
-// blocks each CTA enciphers.  This variant keeps each of T0..T3
-// (and the inverse S-box) once, 4-5 KiB of shared memory: one word per thread
-// to write.  Its lookups may meet bank conflicts (32 lanes, random bytes, one
-// copy), which costs little when every warp is one of a handful on its SM.
+// AES_KERNEL_TABLE_COMPACT: each of T0..T3 (and the inverse S-box) once, 4-5 KiB of
+// shared memory, one word per thread to write.  Its lookups may meet bank conflicts
+// (32 lanes, random bytes, one copy).  Nothing chooses it by itself any more: with
+// one replicated table of 32 KiB per CTA short calls are faster than with this
+// (AES-128 / 256 encryption, captured calls, this against table_kernel: 1 block
+// 2.01 / 2.24 and 1.90 / 2.08 us, 4,096 blocks 2.40 / 2.72 and 2.10 / 2.28, 9,728 blocks
+// 2.27 / 2.56 and 2.12 / 2.29).
 // Word x of table k sits at byte 1024*k + 4*x; the inverse S-box (its value in
 // all four bytes) follows at 4096.
 
 constexpr uint32_t kCompactWords = 5 * 256;
-
-// AES_KERNEL_TABLE takes the compact tables up to this many blocks per SM.  Measured
-// on the GB300 (AES-128 / 256 encryption, a call in a graph, compact against
-// replicated): 256 blocks 2.71 / 2.69 and 3.02 / 2.87 us, 9,728 blocks 2.63 / 3.04 and
-// 2.98 / 3.24, 13,000 blocks 3.12 / 3.17 and 3.50 / 3.44; in a stream, where fills
-// overlap the call before, 15,000 blocks 3.02 / 3.02 and 3.95 / 3.18.
-constexpr uint64_t kCompactBlocksPerSm = 64;
 
 template <int K>
 __device__ __forceinline__ uint32_t byte4(uint32_t w) {  // 4 * (byte K of w)
@@ -261,10 +255,6 @@ __global__ void __launch_bounds__(256) table_compact_kernel(const EcbArgs a) {
 
 // ------------------------------------------------------------------ launcher
 
-}  // namespace gbaes
-
-namespace gbaes {
-
 namespace {
 
 using KernelFn = void (*)(const EcbArgs);
@@ -272,7 +262,6 @@ using KernelFn = void (*)(const EcbArgs);
 template <int NR, int MODE>
 KernelFn pick_bpt(int bpt) {
     switch (bpt) {
-        case 0: return table_compact_kernel<NR, MODE>;
         case 1: return table_kernel<NR, MODE, 1>;
         case 2: return table_kernel<NR, MODE, 2>;
         case 4: return table_kernel<NR, MODE, 4>;
@@ -281,31 +270,38 @@ KernelFn pick_bpt(int bpt) {
 }
 
 template <int NR>
-KernelFn pick_mode(int mode, int bpt) {
+KernelFn pick_mode(int mode, int bpt, bool compact) {
     switch (mode) {
-        case kEnc: return pick_bpt<NR, kEnc>(bpt);
-        case kDec: return pick_bpt<NR, kDec>(bpt);
-        case kCtr: return pick_bpt<NR, kCtr>(bpt);
-        case kCbcDec: return pick_bpt<NR, kCbcDec>(bpt);
+        case kEnc: return compact ? table_compact_kernel<NR, kEnc> : pick_bpt<NR, kEnc>(bpt);
+        case kDec: return compact ? table_compact_kernel<NR, kDec> : pick_bpt<NR, kDec>(bpt);
+        case kCtr: return compact ? nullptr : pick_bpt<NR, kCtr>(bpt);
+        case kCbcDec: return compact ? nullptr : pick_bpt<NR, kCbcDec>(bpt);
         default: return nullptr;
     }
 }
 
-// bpt 0 selects the compact-table kernel.
-KernelFn pick(int nr, int mode, int bpt) {
+KernelFn pick(int nr, int mode, int bpt, bool compact) {
     switch (nr) {
-        case 10: return pick_mode<10>(mode, bpt);
-        case 12: return pick_mode<12>(mode, bpt);
-        case 14: return pick_mode<14>(mode, bpt);
+        case 10: return pick_mode<10>(mode, bpt, compact);
+        case 12: return pick_mode<12>(mode, bpt, compact);
+        case 14: return pick_mode<14>(mode, bpt, compact);
         default: return nullptr;
     }
 }
 
 }  // namespace
 
-constexpr int kMinThreads = 128;
+// A CTA with less than one pass of blocks keeps at least this many threads, one chunk
+// of its table's pieces each: with 128, which fill in two steps, 13,000 blocks take
+// 2.71 us in a captured call instead of 2.43 (2.06 in a stream instead of 1.98).
+constexpr int kMinThreads = (int)(kFillPieces / kFillChunk);
 
-uint64_t compact_limit_blocks(int sms) { return (uint64_t)sms * kCompactBlocksPerSm; }
+// Up to this many blocks per SM a call runs one CTA on each SM, above it two: a second
+// table to write costs more than the warps of a second CTA give.  Captured calls with two
+// CTAs and with one: 9,728 blocks 2.29 / 2.12 us (AES-256 decryption 2.49 / 2.29), 19,456
+// 2.44 / 2.14 (2.75 / 2.31); at 256 blocks per SM (32,768 blocks) 2.53 / 2.38 (2.83 / 2.64), but
+// in a stream, where the fill overlaps the call before, 2.02 / 2.52 (2.27 / 3.08).
+constexpr uint64_t kOneCtaBlocksPerSm = 128;
 
 int launch_table(EcbArgs a, int nr, Mode mode, int threads, int bpt, int variant, cudaStream_t stream) {
     DeviceInfo info;
@@ -313,19 +309,18 @@ int launch_table(EcbArgs a, int nr, Mode mode, int threads, int bpt, int variant
     if (rc) return rc;
     const uint64_t n = a.nblocks;
     const uint64_t sms = (uint64_t)info.sms;
-    if (variant == AES_KERNEL_TABLE) variant = n <= compact_limit_blocks(info.sms) ? AES_KERNEL_TABLE_COMPACT
-                                                                                   : AES_KERNEL_TABLE_REPLICATED;
-    if (threads == 0 || bpt == 0) {
-        // The automatic shape: one block per thread while that covers the input, which
-        // spreads a short call over the most warps.
-        if (threads == 0) threads = 512;
-        if (bpt == 0) bpt = n <= 2 * sms * (uint64_t)threads ? 1 : 2;
-    }
-    KernelFn fn = pick(nr, mode, variant == AES_KERNEL_TABLE_COMPACT ? 0 : bpt);
+    const bool compact = variant == AES_KERNEL_TABLE_COMPACT;
+    // The automatic shape: one block per thread while that covers the input, which
+    // spreads a short call over the most warps.  The shortest take it whatever shape is
+    // asked for, unless the variant is too.
+    if (variant == AES_KERNEL_TABLE && n <= kOneCtaBlocksPerSm * sms) threads = bpt = 0;
+    if (threads == 0) threads = 512;
+    if (bpt == 0) bpt = n <= 2 * sms * (uint64_t)threads ? 1 : 2;
+    KernelFn fn = pick(nr, mode, bpt, compact);
     if (!fn) return fail(AES_ERR_ARG, "no table kernel for nr=%d mode=%d blocks_per_thread=%d", nr, (int)mode, bpt);
     unsigned grid;
     int smem = 0;
-    if (variant == AES_KERNEL_TABLE_COMPACT) {
+    if (compact) {
         // A warp per 32 blocks, spread over the SMs (at most 8 warps per CTA, 8 CTAs per SM).
         const uint64_t warps = (n + 31) / 32;
         uint64_t per_cta = (warps + sms - 1) / sms;
@@ -334,20 +329,21 @@ int launch_table(EcbArgs a, int nr, Mode mode, int threads, int bpt, int variant
         grid = (unsigned)(ctas < 8 * sms ? ctas : 8 * sms);
         threads = (int)(32 * per_cta);
     } else {
-        // Two CTAs per SM (64 registers a thread), one above 512 threads.
-        const uint64_t ctas = threads <= 512 ? 2 * sms : sms;
+        // Two CTAs per SM (64 registers a thread); one above 512 threads, and for short
+        // calls if a pass of it covers its blocks.
+        const bool brief = n <= sms * std::min<uint64_t>(kOneCtaBlocksPerSm, (uint64_t)threads);
+        const uint64_t ctas = brief || threads > 512 ? sms : 2 * sms;
         const uint64_t units = (n + 31) / 32;
         grid = (unsigned)(units < ctas ? units : ctas);
-        // A CTA with less than one pass of blocks needs no more threads than those,
-        // but a quick fill wants some.
+        // A CTA with less than one pass of blocks needs no more threads than those.
         const uint64_t share = (units + grid - 1) / grid * 32;
         if (share < (uint64_t)threads) threads = (int)(share < kMinThreads ? std::min(kMinThreads, threads) : (int)share);
-        // With one block per thread (32 registers) four CTAs and more would fit, and a
+        // With one block per thread (40 registers) three CTAs and more would fit, and a
         // call's CTAs, placed while the call before it still runs, would crowd some SMs and
         // leave others idle (65,536 blocks 3.1-4.1 us per call of a stream, 100,000 blocks
         // 3.3-4.5): with this much shared memory two do (2.7, 3.1).
         smem = (int)kTableBytes;
-        if (bpt == 1 && threads <= 512) {
+        if (bpt == 1 && threads <= 512 && !brief) {
             smem = 100 << 10;
             rc = set_max_dynamic_smem((const void*)fn, smem);
             if (rc) return rc;

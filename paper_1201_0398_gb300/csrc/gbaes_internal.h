@@ -76,12 +76,9 @@ struct RangeCache {
 // check_device_range through a cache (nullptr: no cache).
 int check_device_range_cached(const void* p, size_t bytes, const char* what, RangeCache* cache);
 
-// Largest call (in blocks) that AES_KERNEL_TABLE runs with compact tables.
-uint64_t compact_limit_blocks(int sms);
-
-// Launches the T-table kernel (ecb_table.cu).  variant: AES_KERNEL_TABLE (picks
-// by size), AES_KERNEL_TABLE_COMPACT or AES_KERNEL_TABLE_REPLICATED; threads
-// and bpt shape the replicated kernel only.
+// Launches the T-table kernel (ecb_table.cu).  variant: AES_KERNEL_TABLE_COMPACT (ECB
+// only), or AES_KERNEL_TABLE / AES_KERNEL_TABLE_REPLICATED, the replicated kernel,
+// which alone threads and bpt (0: by size) shape.
 int launch_table(EcbArgs a, int nr, Mode mode, int threads, int bpt, int variant, cudaStream_t stream);
 
 // CTR on inputs of at least ctr_min_blocks blocks (ctr.cu); a.first is any 64-bit index.

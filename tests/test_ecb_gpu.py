@@ -408,7 +408,7 @@ def compact_sizes():
 
 @pytest.mark.parametrize("bits", BITS)
 def test_compact_tables_vs_oracle(gbaes, bits):
-    """The compact-table kernel (each table stored once) in every mode."""
+    """The compact-table kernel (each table stored once), and short CTR and CBC calls."""
     rng = np.random.default_rng(1300 + bits)
     key = rng.integers(0, 256, bits // 8, dtype=np.uint8).tobytes()
     iv = rng.integers(0, 256, 16, dtype=np.uint8).tobytes()
@@ -419,7 +419,7 @@ def test_compact_tables_vs_oracle(gbaes, bits):
         for decrypt in (False, True):
             out = gbaes.ecb_ex(k, x, decrypt=decrypt, kernel=gbaes.KERNEL_TABLE_COMPACT)
             assert np.array_equal(host(out), oracle.ecb(key, bits, data, decrypt=decrypt)), (n, decrypt)
-        if n <= 128 * sms():  # CTR and CBC decryption take the compact tables for calls this small
+        if n <= 128 * sms():  # (CTR and CBC decryption have the replicated table only)
             for kind in (oracle.CTR_BE128, oracle.CTR_LE32_CARRY):
                 assert np.array_equal(host(gbaes.ctr_xcrypt(k, iv, x, kind=kind)),
                                       oracle.ctr(key, bits, iv, data, kind)), (n, kind)
@@ -429,10 +429,9 @@ def test_compact_tables_vs_oracle(gbaes, bits):
 
 @pytest.mark.parametrize("decrypt", (False, True))
 def test_size_dispatch_and_balanced_shapes_vs_oracle(gbaes, decrypt):
-    """AES_KERNEL_TABLE picks compact tables for small calls and the replicated
-    tables above; the replicated kernel shrinks its CTAs so that calls of a few
-    tiles per SM spread evenly.  Sizes on both sides of the switch and across
-    the shrinking range, through the default call and both variants forced."""
+    """AES_KERNEL_TABLE runs one CTA per SM for short calls and two above, and shrinks
+    its CTAs so that calls of a few tiles per SM spread evenly.  Sizes on both sides
+    of the switch and across the shrinking range, through the default call and both variants forced."""
     rng = np.random.default_rng(1400 + decrypt)
     s = sms()
     for bits in (128, 256):
