@@ -149,11 +149,15 @@ __global__ void __launch_bounds__(kCtrThreads, 1) ctr_kernel(const EcbArgs a) {
     }
 }
 
-// Shortest input that takes this kernel: five rows for every row range.  With
-// fewer the two rounds ahead of a range's first row and the uneven last rows cost
-// more than the rounds spared: 311,296 blocks (four rows) 8.28 us in the table kernel,
-// 8.47 here (AES-256 10.34 / 10.75), 400,000 blocks 10.57 / 9.85 (13.48 / 12.76).
-uint64_t ctr_min_blocks(int sms) { return (uint64_t)sms * 2u * 256u * 5u; }
+// Shortest input that takes this kernel: 2.5 rows for every row range, so that half of
+// the ranges have three rows and half two.  With fewer, the two rounds ahead of a range's
+// first row cost more than the rounds spared; from 330,000 to 470,000 blocks the two kernels
+// are within 2% of one another either way, by how the rows and passes divide.  The table
+// kernel against this one, captured calls / calls of a stream, in us: AES-128 272,384
+// blocks 6.98 / 6.09 and 7.14 / 6.65, 389,120 9.16 / 8.42 and 8.82 / 8.36, 544,768 11.81 / 11.10 and
+// 11.03 / 10.61; AES-256 8.81 / 7.88 and 9.16 / 8.69, 11.74 / 10.97 and 11.61 / 11.15, 15.38 / 14.63 and
+// 14.82 / 14.39.
+uint64_t ctr_min_blocks(int sms) { return (uint64_t)sms * kCtrRanges * 256u * 5u / 2u; }
 
 int launch_ctr(EcbArgs a, int nr, cudaStream_t stream) {
     DeviceInfo info;
