@@ -5,6 +5,10 @@ open-loop replay, a producer stopped mid-run, draining and argument errors.
 GPU: every request's output equals the single-message kernel's output for the
 same request alone (and the oracle on a sample), the budget is never exceeded,
 and batches overlap on the device."""
+import ctypes
+import os
+import time
+
 import numpy as np
 import pytest
 
@@ -722,3 +726,57 @@ def test_server_with_payloads_in_page_locked_host_memory(gbaes, resident):
         want = oracle.ecb(raw_keys[k], int(bits[k]), xs[a:a + m], decrypt=bool(reqs["decrypt"][i]), nthreads=1)
         assert np.array_equal(ys[b:b + m], want), i
     assert gbaes.device_status() == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("arrivals", [[0.0, 0.04], [0.0] * 1024 + [0.2], [0.0, 0.2]])
+def test_replay_thread_locks_its_stack_unless_a_burst(gbaes, arrivals):
+    """The top of the replay thread's stack is page-locked while it waits for an
+    arrival, however short the schedule (its pages cannot be moved under it), and
+    every request of schedules and bursts comes out."""
+
+    def replay_stack_pointer():
+        for tid in os.listdir("/proc/self/task"):
+            try:
+                if open(f"/proc/self/task/{tid}/comm").read().strip() == "gbaes-replay":
+                    f = open(f"/proc/self/task/{tid}/syscall").read().split()
+                    if len(f) == 9:  # (blocked in a system call: number, six arguments, stack pointer, program counter)
+                        return int(f[7], 16)
+            except OSError as e:
+                if e.errno in (1, 13):
+                    pytest.skip("/proc/<pid>/task/<tid>/syscall cannot be read here")
+        return None
+
+    cuda = ctypes.CDLL("libcuda.so.1")
+    kind = ctypes.c_uint()
+    key = bytes(range(16))
+    n = len(arrivals)
+    x = torch.randint(0, 256, (16 * n,), dtype=torch.uint8, device="cuda")
+    y = torch.zeros_like(x)
+    r = np.zeros(n, gbaes.REQUEST)
+    r["id"] = np.arange(n)
+    r["in_ptr"] = x.data_ptr() + 16 * np.arange(n)
+    r["out_ptr"] = y.data_ptr() + 16 * np.arange(n)
+    r["nblocks"] = 1
+    r["arrival_s"] = arrivals
+    torch.cuda.synchronize()
+    srv = gbaes.Server([gbaes.Key(key)])
+    srv.replay(r)
+    time.sleep(0.01)  # (the thread has begun by then, and waits for the last arrival)
+    sp = replay_stack_pointer()
+    assert sp is not None
+    rc = cuda.cuPointerGetAttribute(ctypes.byref(kind), 2, ctypes.c_uint64(sp))  # CU_POINTER_ATTRIBUTE_MEMORY_TYPE
+    srv.replay_join()
+    srv.drain(10.0)
+    done = srv.poll_all()
+    assert len(done) == n and (done["status"] == 0).all()
+    assert rc == 0 and kind.value == 1  # CU_MEMORYTYPE_HOST: page-locked
+    r["arrival_s"] = 0  # the same as a burst
+    y.zero_()
+    torch.cuda.synchronize()
+    srv.replay(r)
+    srv.replay_join()
+    srv.drain(10.0)
+    assert len(srv.poll_all()) == n
+    srv.close()
+    assert np.array_equal(y.cpu().numpy(), oracle.ecb(key, 128, x.cpu().numpy()))
