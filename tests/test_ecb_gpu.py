@@ -544,6 +544,54 @@ def test_dependent_calls_on_buffers_off_by_a_block(gbaes, n):
     assert gbaes.device_status() == 0
 
 
+@pytest.mark.parametrize("n", (1, 4097, 65_536, 300_001))
+def test_dependent_calls_of_other_kernels_and_streams(gbaes, n):
+    """The bitsliced kernel, the allocation-free batch and the direct host pipeline
+    in chains of calls without a wait on the host, each on its predecessor's output,
+    and the chain handed to the other of two streams by events at every step."""
+    rng = np.random.default_rng(n)
+    raw = [rng.integers(0, 256, b // 8, dtype=np.uint8).tobytes() for b in BITS]
+    ks = [gbaes.Key(r) for r in raw]
+    data = rng.integers(0, 256, 16 * n, dtype=np.uint8)
+    lib = gbaes.load()
+    ctxs = gbaes._ctx_array(ks)
+    cut = n // 3
+    descs = gbaes.make_descs([0, 16 * cut], [0, 16 * cut], [cut, n - cut], [1, 2], [1, 0])
+    x = dev(data)
+    h = torch.empty(16 * n, dtype=torch.uint8, pin_memory=True)
+    pipe = gbaes.Pipeline(mode=gbaes.PIPE_DIRECT)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    steps = 6
+    for i in range(steps):
+        s = streams[i % 2]
+        s.wait_stream(streams[1 - i % 2])
+        with torch.cuda.stream(s):
+            gbaes.encrypt_ecb(ks[i % 3], x, x)
+            gbaes.ecb_ex(ks[(i + 1) % 3], x, x, kernel=gbaes.KERNEL_BITSLICED)
+            gbaes.ecb_ex(ks[(i + 2) % 3], x, x, decrypt=True, kernel=gbaes.KERNEL_BITSLICED)
+            rc = lib.aes_ecb_batch_noalloc(ctypes.c_void_p(descs.ctypes.data), 2, ctxs, 3,
+                                           ctypes.c_void_p(x.data_ptr()), 16 * n, ctypes.c_void_p(x.data_ptr()), 16 * n,
+                                           ctypes.c_void_p(s.cuda_stream))
+            assert rc == 0
+            h.copy_(x, non_blocking=True)
+            pipe.ecb(ks[i % 3], h, h)
+            pipe.ecb(ks[(i + 1) % 3], h, h, decrypt=True)
+            x.copy_(h, non_blocking=True)
+    got = host(x)
+    want = data
+    for i in range(steps):
+        want = oracle.ecb(raw[i % 3], BITS[i % 3], want)
+        want = oracle.ecb(raw[(i + 1) % 3], BITS[(i + 1) % 3], want)
+        want = oracle.ecb(raw[(i + 2) % 3], BITS[(i + 2) % 3], want, decrypt=True)
+        parts = [oracle.ecb(raw[1], 192, want[:16 * cut], decrypt=True)] if cut else []
+        want = np.concatenate(parts + [oracle.ecb(raw[2], 256, want[16 * cut:])])
+        want = oracle.ecb(raw[i % 3], BITS[i % 3], want)
+        want = oracle.ecb(raw[(i + 1) % 3], BITS[(i + 1) % 3], want, decrypt=True)
+    assert np.array_equal(got, want)
+    assert gbaes.device_status() == 0
+
+
 @pytest.mark.parametrize("bits", BITS)
 @pytest.mark.parametrize("captured", (False, True))
 def test_short_calls_in_both_orders(gbaes, bits, captured):

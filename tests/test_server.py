@@ -7,6 +7,7 @@ same request alone (and the oracle on a sample), the budget is never exceeded,
 and batches overlap on the device."""
 import ctypes
 import os
+import re
 import time
 
 import numpy as np
@@ -780,3 +781,46 @@ def test_replay_thread_locks_its_stack_unless_a_burst(gbaes, arrivals):
     assert len(srv.poll_all()) == n
     srv.close()
     assert np.array_equal(y.cpu().numpy(), oracle.ecb(key, 128, x.cpu().numpy()))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("total", ((1 << 16) - 1, 1 << 16, 300_000))
+@pytest.mark.parametrize("shape", ({}, {"threads": 256, "blocks_per_thread": 4}))
+def test_micro_batch_of_open_shape(gbaes, total, shape):
+    """Micro-batches of servers whose shape is left open run 2 blocks per thread from 2^16 blocks on, and 1 below;
+    with a shape given they keep it.  Each burst of 200 requests, one micro-batch or a few, as single calls compute it."""
+    rng = np.random.default_rng(total)
+    n = 200
+    cut = np.sort(rng.choice(np.arange(1, total), n - 1, replace=False))
+    nblocks = np.diff(np.concatenate([[0], cut, [total]]))
+    off = (np.cumsum(nblocks) - nblocks) * 16
+    keys = [gbaes.Key(rng.integers(0, 256, b // 8, dtype=np.uint8).tobytes()) for b in (128, 192, 256) * 5]
+    x = torch.randint(0, 256, (16 * total,), dtype=torch.uint8, device="cuda")
+    y, want = torch.zeros_like(x), torch.zeros_like(x)
+    r = np.zeros(n, gbaes.REQUEST)
+    r["id"] = np.arange(n)
+    r["in_ptr"], r["out_ptr"] = x.data_ptr() + off, y.data_ptr() + off
+    r["nblocks"], r["key_index"], r["decrypt"] = nblocks, rng.integers(0, len(keys), n), rng.integers(0, 2, n)
+    for i in range(n):
+        a, b = int(off[i]), int(off[i] + 16 * nblocks[i])
+        (gbaes.decrypt_ecb if r["decrypt"][i] else gbaes.encrypt_ecb)(keys[r["key_index"][i]], x[a:b], want[a:b])
+    torch.cuda.synchronize()
+    srv = gbaes.Server(keys, **shape)
+    for _ in range(3):  # (until the profiler, as it starts, has missed no launch)
+        y.zero_()
+        torch.cuda.synchronize()
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            srv.replay(r)
+            srv.replay_join()
+            srv.drain(20.0)
+            torch.cuda.synchronize()
+        done = srv.poll_all()
+        assert len(done) == n and (done["status"] == 0).all()
+        assert torch.equal(y, want)
+        bpts = {int(m[1]) for e in prof.events() for m in [re.search(r"batch_kernel<(\d)", e.name)] if m}
+        if bpts:
+            break
+    srv.close()
+    if len(np.unique(done["launch_s"])) == 1:  # all of it in one micro-batch
+        assert bpts == {shape.get("blocks_per_thread", 2 if total >= 1 << 16 else 1)}
+    assert gbaes.device_status() == 0
