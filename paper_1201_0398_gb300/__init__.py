@@ -29,6 +29,7 @@ __all__ = [
     "cbc_decrypt",
     "set_kernel",
     "set_tuning",
+    "tuning",
     "device_status",
     "key_schedule",
     "host_tables",

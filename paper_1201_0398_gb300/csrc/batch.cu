@@ -529,7 +529,8 @@ static int plan_launch_args(aes_batch_plan* P, const void* in_base, size_t in_by
 // units per warp, up to kJoinMax blocks and a kJoinPerMsg-th of the mean message
 // (messages up to 4 MiB, 512 x 8: 3.37 GB 4,285 us with tiles of 512 blocks one at a
 // time, 4,246 with 1,024 blocks, 4,234 with 2,048, 4,230 with 4,096; 10,000 messages up
-// to 256 KiB, 1,700 blocks on average, 271 MB: 382 with 512, 398 with 1,024, 455 with 2,048).
+// to 256 KiB, 1,700 blocks on average, 271 MB: 382 with 512, 398 with 1,024, 455 with 2,048;
+// here and below as measured before crossing passes ran 4 blocks at a time).
 constexpr uint64_t kTilesPerWarp = 4;
 constexpr uint64_t kPartsPerWarp = 8;
 constexpr uint64_t kJoinMax = 2048;  // blocks

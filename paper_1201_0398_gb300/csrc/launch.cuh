@@ -7,8 +7,8 @@
 // may start while its predecessor still runs or drains: it fills its shared-memory
 // tables, which depend on no earlier work, and then waits (pdl_wait) for everything
 // before it in the stream to have ended and its writes to be visible.  Measured on a
-// stream of such calls, before and after: 4 KiB 4.10 -> 2.6 us (host bound), 1 MiB 6.15 ->
-// 2.75, 9 MiB 15.8 -> 12.0, 64 MiB 79.9 -> 74.6.  Filling the tables before the wait
+// stream of such calls, before and after: 4 KiB 4.10 -> 1.9 us (host bound), 1 MiB 6.15 ->
+// 2.4, 9 MiB 15.8 -> 11.8, 64 MiB 79.9 -> 74.6.  Filling the tables before the wait
 // instead of after it is 0.7 us of that.  Where there is no predecessor to wait for,
 // the fill would only keep the first blocks' loads waiting (4 KiB in a captured graph
 // 2.32 us with the loads first, 2.46 with the fill first; up to 300 KiB 0.12-0.2 us):
